@@ -289,6 +289,8 @@ struct MlpModel {
     float* Hh = nullptr;
     float* Z = nullptr;
     float* dZ = nullptr;
+    float* part = nullptr;   // batch statistics and slices of the weight gradients
+    size_t part_bytes = 0;
     float* loss = nullptr;
     // BF16 inference images (swizzled operand layouts), rebuilt when stale
     void* img = nullptr;

@@ -29,10 +29,22 @@
 namespace knng {
 
 // ---------------------------------------------------------------------------
-// Tiled FP32 GEMM: C[M][N] (+)= sum_k A(m, k) B(k, n) with A(m, k) = TA ?
+// Tiled FP32 GEMM: C[M][N] = sum_k A(m, k) B(k, n) with A(m, k) = TA ?
 // A[k*lda + m] : A[m*lda + k] and B(k, n) = TB ? B[n*ldb + k] : B[k*ldb + n].
 // Epilogue: EPI 0 plain store, 1 = + bias[n], store pre-activation to aux and
-// GELU to C, 2 = + bias[n], 3 = tanh(. + bias[n]).
+// GELU to C, 3 = tanh(. + bias[n]), 4 = times GELU'(aux) (the backward pass
+// through the activation), 5 = one K slice of a reduction: slice z of K
+// (kper entries) goes to C + z * (M*N + M), followed by the slice's row sums
+// of A(m, .) (the bias gradient), for grad_reduce_kernel.
+//
+// A thread block holds a TM x TN tile, 256 threads of (TM/16) x (TN/16)
+// entries each; the next K step of 32 is loaded into registers while the
+// current one is multiplied from shared memory.  TM = 16 / TN = 16 serve the
+// network's 16 or 32 outputs, where a 64-wide tile would be mostly padding.
+// The weight gradients contract over the batch (K = 8192 rows of a
+// 4,096-edge batch against 256 x 96 outputs): without the K slices 8 blocks
+// did the whole contraction (2.1 ms each of the two on GB300; 11 us with
+// slices over about two blocks per SM).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ float gelu_f(float a)
 {
@@ -43,70 +55,129 @@ __device__ __forceinline__ float gelu_grad_f(float a)
     return 0.5f * (1.0f + erff(a * 0.70710678118654752f)) + a * 0.39894228040143268f * __expf(-0.5f * a * a);
 }
 
-template <bool TA, bool TB, int EPI>
-__global__ void __launch_bounds__(256) gemm_kernel(int M, int N, int K, const float* __restrict__ A, int lda,
+constexpr int kGemmTK = 32;
+
+template <bool TA, bool TB, int EPI, int TM, int TN>
+__global__ void __launch_bounds__(256) gemm_kernel(int M, int N, int K, int kper, const float* __restrict__ A, int lda,
                                                    const float* __restrict__ B, int ldb, float* __restrict__ C,
                                                    int ldc, const float* __restrict__ bias, float* __restrict__ aux)
 {
-    constexpr int TM = 64, TN = 64, TK = 16;
+    constexpr int TK = kGemmTK, RM = TM / 16, RN = TN / 16;
+    constexpr int LA = TM * TK / 256, LB = TN * TK / 256;
     __shared__ float As[TK][TM + 4];
     __shared__ float Bs[TK][TN + 4];
     const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
     const int m0 = blockIdx.y * TM, n0 = blockIdx.x * TN;
-    float acc[4][4] = {};
-    for (int k0 = 0; k0 < K; k0 += TK) {
-        for (int e = tid; e < TM * TK; e += 256) {
+    const int kbeg = blockIdx.z * kper, kend = min(K, kbeg + kper);
+    float acc[RM][RN] = {};
+    float rsum[RM] = {};
+    float ra[LA], rb[LB];
+    auto fetch = [&](int k0) {
+#pragma unroll
+        for (int i = 0; i < LA; ++i) {
+            const int e = tid + 256 * i;
             const int mm = TA ? e % TM : e / TK, kk = TA ? e / TM : e % TK;
             const int m = m0 + mm, k = k0 + kk;
-            As[kk][mm] = (m < M && k < K) ? (TA ? A[(int64_t)k * lda + m] : A[(int64_t)m * lda + k]) : 0.f;
+            ra[i] = (m < M && k < kend) ? (TA ? A[(int64_t)k * lda + m] : A[(int64_t)m * lda + k]) : 0.f;
         }
-        for (int e = tid; e < TN * TK; e += 256) {
+#pragma unroll
+        for (int i = 0; i < LB; ++i) {
+            const int e = tid + 256 * i;
             const int nn = TB ? e / TK : e % TN, kk = TB ? e % TK : e / TN;
             const int n = n0 + nn, k = k0 + kk;
-            Bs[kk][nn] = (n < N && k < K) ? (TB ? B[(int64_t)n * ldb + k] : B[(int64_t)k * ldb + n]) : 0.f;
+            rb[i] = (n < N && k < kend) ? (TB ? B[(int64_t)n * ldb + k] : B[(int64_t)k * ldb + n]) : 0.f;
+        }
+    };
+    fetch(kbeg);
+    for (int k0 = kbeg; k0 < kend; k0 += TK) {
+        if (k0 > kbeg) __syncthreads();
+#pragma unroll
+        for (int i = 0; i < LA; ++i) {
+            const int e = tid + 256 * i;
+            As[TA ? e / TM : e % TK][TA ? e % TM : e / TK] = ra[i];
+        }
+#pragma unroll
+        for (int i = 0; i < LB; ++i) {
+            const int e = tid + 256 * i;
+            Bs[TB ? e % TK : e / TN][TB ? e / TK : e % TN] = rb[i];
         }
         __syncthreads();
+        if (k0 + TK < kend) fetch(k0 + TK);
 #pragma unroll
         for (int kk = 0; kk < TK; ++kk) {
-            float a[4], b[4];
+            float a[RM], b[RN];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = As[kk][ty * 4 + i];
+            for (int i = 0; i < RM; ++i) a[i] = As[kk][ty * RM + i];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx * 4 + j];
+            for (int j = 0; j < RN; ++j) b[j] = Bs[kk][tx * RN + j];
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int i = 0; i < RM; ++i) {
 #pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+                for (int j = 0; j < RN; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+                if (EPI == 5) rsum[i] += a[i];
+            }
         }
-        __syncthreads();
     }
+    if (EPI == 5) C += (int64_t)blockIdx.z * ((int64_t)M * N + M);
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < RM; ++i) {
+        const int m = m0 + ty * RM + i;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int m = m0 + ty * 4 + i, n = n0 + tx * 4 + j;
+        for (int j = 0; j < RN; ++j) {
+            const int n = n0 + tx * RN + j;
             if (m >= M || n >= N) continue;
             float v = acc[i][j];
             if (EPI == 1) {
                 v += bias[n];
                 aux[(int64_t)m * ldc + n] = v;
                 v = gelu_f(v);
-            } else if (EPI == 2) {
-                v += bias[n];
             } else if (EPI == 3) {
                 v = tanhf(v + bias[n]);
+            } else if (EPI == 4) {
+                v *= gelu_grad_f(aux[(int64_t)m * ldc + n]);
             }
             C[(int64_t)m * ldc + n] = v;
         }
+        if (EPI == 5 && blockIdx.x == 0 && tx == 0 && m < M) C[(int64_t)M * N + m] = rsum[i];
+    }
 }
 
-template <bool TA, bool TB, int EPI>
-static void gemm(int M, int N, int K, const float* A, int lda, const float* B, int ldb, float* C, int ldc,
+template <bool TA, bool TB, int EPI, int TM, int TN>
+static void gemm(int M, int N, int K, int kper, const float* A, int lda, const float* B, int ldb, float* C, int ldc,
                  const float* bias, float* aux, cudaStream_t st)
 {
-    dim3 grid((N + 63) / 64, (M + 63) / 64);
-    gemm_kernel<TA, TB, EPI><<<grid, 256, 0, st>>>(M, N, K, A, lda, B, ldb, C, ldc, bias, aux);
+    dim3 grid((N + TN - 1) / TN, (M + TM - 1) / TM, (K + kper - 1) / kper);
+    gemm_kernel<TA, TB, EPI, TM, TN><<<grid, 256, 0, st>>>(M, N, K, kper, A, lda, B, ldb, C, ldc, bias, aux);
     note_launches(1);
+}
+
+// K entries per slice of a weight-gradient contraction: about two blocks per
+// SM over the output tiles and slices, whole K steps, at least four of them.
+static int slice_len(int tiles, int K)
+{
+    const int slices = std::max(1, 2 * num_sms() / std::max(1, tiles));
+    const int len = (K + slices - 1) / slices;
+    return std::max(4 * kGemmTK, (len + kGemmTK - 1) / kGemmTK * kGemmTK);
+}
+
+// Packed gradient from the slices: entry e of the first c1 (W1 | b1) sums its
+// s1 slices, the rest (W2 | b2, c2 entries) its s2.
+__global__ void grad_reduce_kernel(int c1, int s1, const float* __restrict__ p1, int c2, int s2,
+                                   const float* __restrict__ p2, float* __restrict__ g)
+{
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= c1 + c2) return;
+    const bool first = e < c1;
+    const float* p = first ? p1 + e : p2 + (e - c1);
+    const int c = first ? c1 : c2, s = first ? s1 : s2;
+    // four running sums keep four loads in flight
+    float a[4] = {0.f, 0.f, 0.f, 0.f};
+    int z = 0;
+    for (; z + 4 <= s; z += 4)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) a[q] += p[(int64_t)(z + q) * c];
+    for (; z < s; ++z) a[0] += p[(int64_t)z * c];
+    g[e] = (a[0] + a[1]) + (a[2] + a[3]);
 }
 
 // ---------------------------------------------------------------------------
@@ -140,143 +211,197 @@ __global__ void sample_batch_kernel(RowLoader<kDT> L, int64_t n, const int32_t* 
 }
 
 // ---------------------------------------------------------------------------
-// Loss and dL/dZ through the batch statistics (one block).  Z: N x C rows,
-// N = 2B.  Writes the loss to *loss and the gradient to dZ.
+// Loss and dL/dZ through the batch statistics.  Z: N x C rows, N = 2B.
+// Four passes over blocks of kLossRows rows (one block did it all before:
+// 0.7 ms of an 8192 x 16 batch, now 12 us): column sums; centred second
+// moments and the pairs' differences; the statistics and the loss (one
+// block, sums of the row blocks in FP64); the gradient.
+//   K = corr, S = (z - mean) / sqrt(var + eps), dS = (2/N) S G with
+//   G = 2 lam offdiag(K).  S has zero column means, so mean(dS) = 0 and
+//   mean(dS_c S_c) = (2/N) sum_{a != c} 2 lam K_ac^2: no pass over the rows
+//   is needed for them.
 // ---------------------------------------------------------------------------
-constexpr int kLossThreads = 1024;
+constexpr int kLossRows = 128;
+constexpr int kLossTile = 32;  // rows summed in FP32 before the FP64 sum
 
-__global__ void __launch_bounds__(kLossThreads) loss_kernel(const float* __restrict__ Z, int N, int C, float lam,
-                                                            float eps, float mus, float* __restrict__ dZ,
-                                                            float* __restrict__ loss)
+// sums[block][C]
+__global__ void __launch_bounds__(256) loss_sum_kernel(const float* __restrict__ Z, int N, int C,
+                                                       double* __restrict__ sums)
 {
-    extern __shared__ float sh[];
-    float* mu = sh;               // C
-    float* var = mu + C;          // C
-    float* P = var + C;           // C
-    float* Kc = P + C;            // C*C
-    float* m1 = Kc + C * C;       // C
-    float* m2 = m1 + C;           // C
-    float* red = m2 + C;          // kLossThreads
-    const int tid = threadIdx.x;
-    const int B = N / 2;
-    // per-column reductions: thread t handles column t % C over rows r = t / C, ...
-    const int per = kLossThreads / C;  // threads per column (C divides 1024)
-    const int c = tid % C, r0 = tid / C;
-    auto col_reduce = [&](float v) -> float {
-        red[tid] = v;
-        __syncthreads();
-        float s = 0.f;
-        if (tid < C)
-            for (int q = 0; q < per; ++q) s += red[q * C + tid];
-        __syncthreads();
-        return s;  // valid for tid < C
-    };
-    float s = 0.f;
-    for (int r = r0; r < N; r += per) s += Z[(int64_t)r * C + c];
-    s = col_reduce(s);
-    if (tid < C) mu[tid] = s / N;
+    __shared__ double red[256];
+    const int tid = threadIdx.x, c = tid % C, per = 256 / C;
+    const int rend = min(N, ((int)blockIdx.x + 1) * kLossRows);
+    double s = 0.0;
+    for (int r = blockIdx.x * kLossRows + tid / C; r < rend; r += per) s += (double)Z[(int64_t)r * C + c];
+    red[tid] = s;
     __syncthreads();
-    float sv = 0.f, sp = 0.f;
-    for (int r = r0; r < N; r += per) {
-        const float zc = Z[(int64_t)r * C + c] - mu[c];
-        sv += zc * zc;
-        if (r < B) {
-            const float dd = Z[(int64_t)r * C + c] - Z[(int64_t)(r + B) * C + c];
-            sp += dd * dd;
+    if (tid < C) {
+        for (int q = 1; q < per; ++q) s += red[q * C + tid];
+        sums[(int64_t)blockIdx.x * C + tid] = s;
+    }
+}
+
+__device__ __forceinline__ void loss_means(const double* __restrict__ sums, int nblk, int N, int C, float* mu)
+{
+    const int lane = threadIdx.x & 31;
+    for (int c = threadIdx.x >> 5; c < C; c += blockDim.x >> 5) {
+        double s = 0.0;
+        for (int b = lane; b < nblk; b += 32) s += sums[(int64_t)b * C + c];
+        for (int o = 16; o >= 1; o >>= 1) s += __shfl_xor_sync(KNNG_FULL_MASK, s, o);
+        if (lane == 0) mu[c] = (float)(s / N);
+    }
+}
+
+// mom[block][C*C + C]: sums of z_a z_b (centred) and of the squared
+// differences of the block's edges.
+__global__ void __launch_bounds__(256) loss_moment_kernel(const float* __restrict__ Z, int N, int C,
+                                                          const double* __restrict__ sums, double* __restrict__ mom)
+{
+    __shared__ float mu[32];
+    __shared__ float zt[kLossTile][33];
+    __shared__ float dt[kLossTile][33];
+    const int tid = threadIdx.x, B = N / 2;
+    loss_means(sums, gridDim.x, N, C, mu);
+    __syncthreads();
+    double acc[4] = {0.0, 0.0, 0.0, 0.0};
+    double accp = 0.0;
+    const int rbeg = blockIdx.x * kLossRows, rend = min(N, rbeg + kLossRows);
+    const int pairs = C * C;  // 256 or 1024: one or four per thread
+    for (int t0 = rbeg; t0 < rend; t0 += kLossTile) {
+        __syncthreads();
+        for (int e = tid; e < kLossTile * C; e += 256) {
+            const int r = t0 + e / C, c = e % C;
+            const float z = r < rend ? Z[(int64_t)r * C + c] : mu[c];
+            const float dd = (r < rend && r < B) ? z - Z[(int64_t)(r + B) * C + c] : 0.f;
+            zt[e / C][c] = z - mu[c];
+            dt[e / C][c] = dd;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int pr = tid + 256 * q;
+            if (pr < pairs) {
+                const int a = pr / C, b = pr % C;
+                float s = 0.f;
+#pragma unroll 8
+                for (int r = 0; r < kLossTile; ++r) s = fmaf(zt[r][a], zt[r][b], s);
+                acc[q] += (double)s;
+            }
+        }
+        if (tid < C) {
+            float s = 0.f;
+#pragma unroll 8
+            for (int r = 0; r < kLossTile; ++r) s = fmaf(dt[r][tid], dt[r][tid], s);
+            accp += (double)s;
         }
     }
-    sv = col_reduce(sv);
-    if (tid < C) var[tid] = sv / N;
-    sp = col_reduce(sp);
-    if (tid < C) P[tid] = sp / B;
-    __syncthreads();
-    // correlation matrix: pair (a, b) of columns, threads split the rows
-    const int pairs = C * C;
-    const int tpp = kLossThreads / pairs > 0 ? kLossThreads / pairs : 1;
-    for (int pr = tid / tpp; pr < pairs; pr += kLossThreads / tpp) {
-        const int a = pr / C, bb = pr % C;
-        const float sa = rsqrtf(var[a] + eps), sb = rsqrtf(var[bb] + eps);
-        float acc = 0.f;
-        for (int r = tid % tpp; r < N; r += tpp)
-            acc += (Z[(int64_t)r * C + a] - mu[a]) * sa * (Z[(int64_t)r * C + bb] - mu[bb]) * sb;
-        // tpp divides 32: reduce inside the thread group
-        for (int o = tpp / 2; o >= 1; o >>= 1) acc += __shfl_down_sync(KNNG_FULL_MASK, acc, o, tpp);
-        if (tid % tpp == 0) Kc[pr] = acc / N;
+    double* o = mom + (int64_t)blockIdx.x * (pairs + C);
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        if (tid + 256 * q < pairs) o[tid + 256 * q] = acc[q];
+    if (tid < C) o[pairs + tid] = accp;
+}
+
+// stats: mean[C] | var[C] | P[C] | K[C*C] (floats), and the loss.
+__global__ void __launch_bounds__(1024) loss_stats_kernel(int N, int C, int nblk, float lam, float eps, float mus,
+                                                          const double* __restrict__ sums,
+                                                          const double* __restrict__ mom, float* __restrict__ stats,
+                                                          float* __restrict__ loss)
+{
+    __shared__ double var[32], P[32], part[32];
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int pairs = C * C, tot = pairs + C;
+    float* Kc = stats + 3 * C;
+    loss_means(sums, nblk, N, C, stats);
+    // the diagonal and the differences first: a warp per column
+    for (int c = w; c < C; c += 32) {
+        double sv = 0.0, sp = 0.0;
+        for (int b = lane; b < nblk; b += 32) {
+            sv += mom[(int64_t)b * tot + c * C + c];
+            sp += mom[(int64_t)b * tot + pairs + c];
+        }
+        for (int o = 16; o >= 1; o >>= 1) {
+            sv += __shfl_xor_sync(KNNG_FULL_MASK, sv, o);
+            sp += __shfl_xor_sync(KNNG_FULL_MASK, sp, o);
+        }
+        if (lane == 0) {
+            var[c] = sv / N;
+            P[c] = sp / (N / 2);
+            stats[C + c] = (float)var[c];
+            stats[2 * C + c] = (float)P[c];
+        }
     }
+    __syncthreads();
+    // correlations: 1024 / pairs threads per pair, neighbours in the block
+    // sums' order so that a warp's loads are contiguous
+    double off = 0.0;
+    __shared__ double seg[1024];
+    const int grp = 1024 / pairs, pr = tid % pairs, g0 = tid / pairs;
+    double s = 0.0;
+    for (int b = g0; b < nblk; b += grp) s += mom[(int64_t)b * tot + pr];
+    seg[tid] = s;
+    __syncthreads();
+    if (tid < pairs) {
+        for (int q = 1; q < grp; ++q) s += seg[q * pairs + tid];
+        const int a = tid / C, b = tid % C;
+        const double k = s / N / sqrt((var[a] + eps) * (var[b] + eps));
+        Kc[tid] = (float)k;
+        if (a != b) off = k * k;
+    }
+    for (int o = 16; o >= 1; o >>= 1) off += __shfl_xor_sync(KNNG_FULL_MASK, off, o);
+    if (lane == 0) part[w] = off;
     __syncthreads();
     if (tid == 0) {
-        float L = 0.f;
-        for (int a = 0; a < C; ++a) L += P[a] / (var[a] + eps);
-        float Ld = 0.f;
-        for (int a = 0; a < C; ++a)
-            for (int bb = 0; bb < C; ++bb)
-                if (a != bb) Ld += Kc[a * C + bb] * Kc[a * C + bb];
-        float Ls = 0.f;
-        for (int a = 0; a < C; ++a) Ls += (1.f - var[a]) * (1.f - var[a]);
-        *loss = L + lam * Ld + mus * Ls;
-    }
-    // dS = (2/N) S G with G = 2 lam offdiag(K); then the column means
-    float d1 = 0.f, d2 = 0.f;
-    for (int r = r0; r < N; r += per) {
-        float ds = 0.f;
+        double L = 0.0, Ld = 0.0, Ls = 0.0;
         for (int a = 0; a < C; ++a) {
-            if (a == c) continue;
-            const float sa = (Z[(int64_t)r * C + a] - mu[a]) * rsqrtf(var[a] + eps);
-            ds += sa * 2.f * lam * Kc[a * C + c];
+            L += P[a] / (var[a] + eps);
+            Ls += (1.0 - var[a]) * (1.0 - var[a]);
         }
-        ds *= 2.f / N;
-        const float sc = (Z[(int64_t)r * C + c] - mu[c]) * rsqrtf(var[c] + eps);
-        d1 += ds;
-        d2 += ds * sc;
+        for (int q = 0; q < 32; ++q) Ld += part[q];
+        *loss = (float)(L + lam * Ld + mus * Ls);
     }
-    d1 = col_reduce(d1);
-    if (tid < C) m1[tid] = d1 / N;
-    d2 = col_reduce(d2);
-    if (tid < C) m2[tid] = d2 / N;
+}
+
+// dL/dZ of every entry, taken through the output tanh: dZpre = dZ (1 - Z^2).
+__global__ void __launch_bounds__(256) loss_grad_kernel(const float* __restrict__ Z, int N, int C, float lam, float eps,
+                                                        float mus, const float* __restrict__ stats,
+                                                        float* __restrict__ dZ)
+{
+    __shared__ float mu[32], isig[32], P[32], var[32], m2[32];
+    __shared__ float Kc[32 * 33];
+    __shared__ float st[256];
+    const int tid = threadIdx.x, B = N / 2;
+    for (int e = tid; e < C * C; e += 256) Kc[(e / C) * 33 + e % C] = stats[3 * C + e];
+    if (tid < C) {
+        mu[tid] = stats[tid];
+        var[tid] = stats[C + tid];
+        P[tid] = stats[2 * C + tid];
+        isig[tid] = 1.f / sqrtf(var[tid] + eps);
+    }
     __syncthreads();
-    for (int r = r0; r < N; r += per) {
-        const float ve = var[c] + eps;
-        const float sig = sqrtf(ve);
-        const float zc = Z[(int64_t)r * C + c] - mu[c];
-        float g = (-P[c] / (ve * ve) - 2.f * mus * (1.f - var[c])) * (2.f / N) * zc;
-        const int rb = r < B ? r : r - B;
-        const float dd = Z[(int64_t)rb * C + c] - Z[(int64_t)(rb + B) * C + c];
-        g += (r < B ? 1.f : -1.f) * (1.f / ve) * (2.f / B) * dd;
-        float ds = 0.f;
-        for (int a = 0; a < C; ++a) {
-            if (a == c) continue;
-            const float sa = (Z[(int64_t)r * C + a] - mu[a]) * rsqrtf(var[a] + eps);
-            ds += sa * 2.f * lam * Kc[a * C + c];
-        }
-        ds *= 2.f / N;
-        const float sc = zc / sig;
-        g += (ds - m1[c] - sc * m2[c]) / sig;
-        dZ[(int64_t)r * C + c] = g;
+    if (tid < C) {
+        float s = 0.f;
+        for (int a = 0; a < C; ++a)
+            if (a != tid) s = fmaf(Kc[a * 33 + tid], Kc[a * 33 + tid], s);
+        m2[tid] = 2.f * lam * s * (2.f / N);
     }
-}
-
-// through the output tanh: dZpre = dZ (1 - Z^2)
-__global__ void tanh_back_kernel(int64_t count, const float* __restrict__ Z, float* __restrict__ dZ)
-{
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < count; e += (int64_t)gridDim.x * blockDim.x)
-        dZ[e] *= 1.f - Z[e] * Z[e];
-}
-
-// dA = dH * GELU'(A)
-__global__ void gelu_back_kernel(int64_t count, const float* __restrict__ A, float* __restrict__ dH)
-{
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < count; e += (int64_t)gridDim.x * blockDim.x)
-        dH[e] *= gelu_grad_f(A[e]);
-}
-
-// column sums: out[n] = sum_m X[m][n]
-__global__ void colsum_kernel(int M, int N, const float* __restrict__ X, float* __restrict__ out)
-{
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
-    float s = 0.f;
-    for (int m = 0; m < M; ++m) s += X[(int64_t)m * N + n];
-    out[n] = s;
+    const int c = tid % C, rl = tid / C, per = 256 / C;
+    const int r = blockIdx.x * per + rl;
+    const float z = r < N ? Z[(int64_t)r * C + c] : mu[c];
+    const float zc = z - mu[c];
+    st[tid] = zc * isig[c];  // S of the block's rows
+    __syncthreads();
+    if (r >= N) return;
+    const float ve = var[c] + eps;
+    float g = (-P[c] / (ve * ve) - 2.f * mus * (1.f - var[c])) * (2.f / N) * zc;
+    const float other = Z[(int64_t)(r < B ? r + B : r - B) * C + c];
+    g += (1.f / ve) * (2.f / B) * (z - other);
+    float ds = 0.f;
+    for (int a = 0; a < C; ++a)
+        if (a != c) ds = fmaf(st[rl * C + a], 2.f * lam * Kc[a * 33 + c], ds);
+    ds *= 2.f / N;
+    g += (ds - st[tid] * m2[c]) * isig[c];
+    dZ[(int64_t)r * C + c] = g * (1.f - z * z);
 }
 
 // Adam step on the packed parameters.
@@ -298,8 +423,42 @@ __global__ void adam_kernel(int count, float* __restrict__ w, const float* __res
 // ---------------------------------------------------------------------------
 constexpr float kLam = 0.05f, kEps = 1e-4f, kSpread = 1.0f;
 
+// Sizes of one batch's scratch: row blocks of the loss, length and number of
+// the K slices of the two weight gradients, entries per slice.
+struct GradScratch {
+    int nblk, k1, s1, c1, k2, s2, c2;
+    size_t bytes;
+};
+static GradScratch grad_scratch(const MlpModel* M, int N)
+{
+    GradScratch g;
+    const int d = M->d, H = M->H, C = M->C;
+    g.nblk = (N + kLossRows - 1) / kLossRows;
+    g.k1 = slice_len(((H + 63) / 64) * ((d + 63) / 64), N);
+    g.s1 = (N + g.k1 - 1) / g.k1;
+    g.c1 = H * d + H;
+    g.k2 = slice_len(((C + 15) / 16) * ((H + 63) / 64), N);
+    g.s2 = (N + g.k2 - 1) / g.k2;
+    g.c2 = C * H + C;
+    g.bytes = sizeof(double) * (size_t)g.nblk * (C * C + 2 * C) +
+              sizeof(float) * (3 * (size_t)C + (size_t)C * C + (size_t)g.s1 * g.c1 + (size_t)g.s2 * g.c2);
+    return g;
+}
+
 static int ensure_rows(MlpModel* M, int rows)
 {
+    // (fewer rows can need a little more: their slices are shorter)
+    const size_t need = grad_scratch(M, rows).bytes;
+    if (need > M->part_bytes) {
+        cudaFree(M->part);
+        M->part = nullptr;
+        M->part_bytes = 0;
+        if (cudaMalloc(&M->part, need) != cudaSuccess) {
+            cudaGetLastError();
+            return KNNG_ERR_OOM;
+        }
+        M->part_bytes = need;
+    }
     if (rows <= M->cap_rows) return KNNG_OK;
     cudaFree(M->Xb);
     cudaFree(M->A);
@@ -324,25 +483,29 @@ static int ensure_rows(MlpModel* M, int rows)
 static cudaError_t loss_grad(MlpModel* M, const float* Xb, int B, cudaStream_t st)
 {
     const int N = 2 * B, d = M->d, H = M->H, C = M->C;
-    gemm<false, true, 1>(N, H, d, Xb, d, M->W1(), d, M->Hh, H, M->b1(), M->A, st);
-    gemm<false, true, 3>(N, C, H, M->Hh, H, M->W2(), H, M->Z, C, M->b2(), nullptr, st);
-    const size_t lsm = sizeof(float) * (6 * C + C * C + kLossThreads);
-    loss_kernel<<<1, kLossThreads, lsm, st>>>(M->Z, N, C, kLam, kEps, kSpread, M->dZ, M->loss);
-    tanh_back_kernel<<<(N * C + 255) / 256, 256, 0, st>>>((int64_t)N * C, M->Z, M->dZ);
-    note_launches(2);
-    float* gW1 = M->g;
-    float* gb1 = gW1 + (int64_t)H * d;
-    float* gW2 = gb1 + H;
-    float* gb2 = gW2 + (int64_t)C * H;
-    gemm<true, false, 0>(C, H, N, M->dZ, C, M->Hh, H, gW2, H, nullptr, nullptr, st);  // dZ^T Hh
-    colsum_kernel<<<(C + 127) / 128, 128, 0, st>>>(N, C, M->dZ, gb2);
-    note_launches(1);
-    gemm<false, false, 0>(N, H, C, M->dZ, C, M->W2(), H, M->Hh, H, nullptr, nullptr, st);  // dH = dZ W2 (into Hh)
-    gelu_back_kernel<<<std::max(1, std::min(num_sms() * 8, (N * H + 255) / 256)), 256, 0, st>>>((int64_t)N * H,
-                                                                                                  M->A, M->Hh);
-    note_launches(1);
-    gemm<true, false, 0>(H, d, N, M->Hh, H, Xb, d, gW1, d, nullptr, nullptr, st);  // dA^T X
-    colsum_kernel<<<(H + 127) / 128, 128, 0, st>>>(N, H, M->Hh, gb1);
+    gemm<false, true, 1, 64, 64>(N, H, d, d, Xb, d, M->W1(), d, M->Hh, H, M->b1(), M->A, st);
+    gemm<false, true, 3, 64, 16>(N, C, H, H, M->Hh, H, M->W2(), H, M->Z, C, M->b2(), nullptr, st);
+    // scratch of this batch: FP64 sums of the row blocks | statistics |
+    // slices of the two weight gradients (sizes: grad_scratch)
+    const GradScratch gs = grad_scratch(M, N);
+    char* base = reinterpret_cast<char*>(M->part);
+    double* sums = reinterpret_cast<double*>(base);
+    double* mom = sums + (size_t)gs.nblk * C;
+    float* stats = reinterpret_cast<float*>(mom + (size_t)gs.nblk * (C * C + C));
+    float* p1 = stats + 3 * C + C * C;
+    float* p2 = p1 + (size_t)gs.s1 * gs.c1;
+    loss_sum_kernel<<<gs.nblk, 256, 0, st>>>(M->Z, N, C, sums);
+    loss_moment_kernel<<<gs.nblk, 256, 0, st>>>(M->Z, N, C, sums, mom);
+    loss_stats_kernel<<<1, 1024, 0, st>>>(N, C, gs.nblk, kLam, kEps, kSpread, sums, mom, stats, M->loss);
+    loss_grad_kernel<<<(N + 256 / C - 1) / (256 / C), 256, 0, st>>>(M->Z, N, C, kLam, kEps, kSpread, stats, M->dZ);
+    note_launches(4);
+    // dW2 = dZ^T Hh and db2, in slices of the batch
+    gemm<true, false, 5, 16, 64>(C, H, N, gs.k2, M->dZ, C, M->Hh, H, p2, H, nullptr, nullptr, st);
+    // dA = (dZ W2) GELU'(A) (into Hh)
+    gemm<false, false, 4, 64, 64>(N, H, C, C, M->dZ, C, M->W2(), H, M->Hh, H, nullptr, M->A, st);
+    // dW1 = dA^T X and db1
+    gemm<true, false, 5, 64, 64>(H, d, N, gs.k1, M->Hh, H, Xb, d, p1, d, nullptr, nullptr, st);
+    grad_reduce_kernel<<<(gs.c1 + gs.c2 + 255) / 256, 256, 0, st>>>(gs.c1, gs.s1, p1, gs.c2, gs.s2, p2, M->g);
     note_launches(1);
     return cudaGetLastError();
 }
@@ -421,7 +584,7 @@ int knng_mlp_destroy(knng_mlp* o)
     cudaGetDevice(&prev);
     cudaSetDevice(M.device);
     cudaDeviceSynchronize();
-    for (float* p : {M.w, M.g, M.am, M.av, M.Xb, M.A, M.Hh, M.Z, M.dZ, M.loss}) cudaFree(p);
+    for (float* p : {M.w, M.g, M.am, M.av, M.Xb, M.A, M.Hh, M.Z, M.dZ, M.part, M.loss}) cudaFree(p);
     cudaFree(M.img);
     cudaSetDevice(prev);
     delete o;
