@@ -318,6 +318,41 @@ __device__ __forceinline__ void warp_bitonic_sort32(uint32_t (&v)[E])
     }
 }
 
+// Batcher's odd-even merge sort on a thread's own registers (191 exchanges of
+// 32 values; the bitonic network has 240), ascending.  Every exchange puts the
+// smaller value at the lower index, so the network of the next power of two
+// without the exchanges past N sorts any N.
+__device__ __forceinline__ void reg_exchange(float& a, float& b)
+{
+    const float lo = fminf(a, b), hi = fmaxf(a, b);
+    a = lo;
+    b = hi;
+}
+__device__ __forceinline__ void reg_exchange(uint64_t& a, uint64_t& b)
+{
+    const bool sw = b < a;
+    const uint64_t lo = sw ? b : a, hi = sw ? a : b;
+    a = lo;
+    b = hi;
+}
+template <class T, int N>
+__device__ __forceinline__ void reg_oddeven_sort(T (&v)[N])
+{
+#pragma unroll
+    for (int p = 1; p < N; p <<= 1) {
+#pragma unroll
+        for (int q = p; q >= 1; q >>= 1) {
+#pragma unroll
+            for (int i = 0; i < N; ++i) {
+                // i starts a pair when it lies in the lower half of a run of
+                // 2q (counted from q mod p) and both ends share a block of 2p
+                const int l = i + q, f = i - (q & (p - 1));
+                if (l < N && f >= 0 && (f & q) == 0 && ((i ^ l) & ~(2 * p - 1)) == 0) reg_exchange(v[i], v[l]);
+            }
+        }
+    }
+}
+
 __device__ __forceinline__ uint32_t lanemask_lt()
 {
     uint32_t m;
@@ -754,18 +789,18 @@ __device__ __forceinline__ float warp_canon_dist32(const RowLoader<kDT>& L, int6
 }
 
 // Rescoring of one row's candidate list (collective over one warp):
-// keys[i * stride], i < nc <= 64, hold (D~, local index j); every candidate
-// is rescored with the canonical FP32 distance between the original rows of
-// lid[self] and lid[j], and the k best by (D, id) go to oi/od (padding -1 /
-// +inf).  ws: kLeafWarpScratch bytes of the warp.
+// cols[i], i < nc <= 64, are local indices j; every candidate is rescored
+// with the canonical FP32 distance between the original rows of lid[self]
+// and lid[j], and the k best by (D, id) go to oi/od (padding -1 / +inf).
+// ws: kLeafWarpScratch bytes of the warp.
 template <int kDT>
-__device__ void leaf_rescore_list(const RowLoader<kDT>& L, const int32_t* lid, int self, const uint64_t* keys,
-                                  int stride, int nc, int k, unsigned char* ws, int32_t* oi, float* od)
+__device__ void leaf_rescore_list(const RowLoader<kDT>& L, const int32_t* lid, int self, const uint16_t* cols,
+                                  int nc, int k, unsigned char* ws, int32_t* oi, float* od)
 {
     const int lane = threadIdx.x & 31;
     int* cid = reinterpret_cast<int*>(ws);                   // 64 point ids
     uint64_t* rk = reinterpret_cast<uint64_t*>(ws + 1024);   // 64 rescored keys
-    for (int c = lane; c < nc; c += 32) cid[c] = lid[(uint32_t)keys[(size_t)c * stride]];
+    for (int c = lane; c < nc; c += 32) cid[c] = lid[cols[c]];
     __syncwarp();
     const int gi = lid[self];
     for (int c0 = 0; c0 < nc; c0 += 16) {

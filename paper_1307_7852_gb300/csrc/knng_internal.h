@@ -179,8 +179,9 @@ std::vector<TcTile> tc_candidates(const TreePlan& P, int d, int prec);
 
 // Staged FP32 rescoring of reduced-precision leaf candidates (one CTA per
 // tree and leaf; the leaf's rows stream through shared memory in 32-entry
-// slices): FP32 rows, 16-byte aligned, k' <= 32, leaves of at most 512.
-bool leaf_rescore_staged_ok(const XDesc& x, int kp, int max_leaf);
+// slices): k' <= 40, leaves of at most 512.  leaf_exact (nullable): leaves to
+// skip.
+bool leaf_rescore_staged_ok(int kp, int max_leaf);
 cudaError_t run_leaf_rescore_staged(const XDesc& x, const TreePlan& P, const DevPlan& dp, int T,
                                     const int32_t* perm, const uint8_t* leaf_exact, const uint16_t* cand, int kp,
                                     int k, int32_t* ids, float* dists, cudaStream_t st);

@@ -58,23 +58,29 @@ static TcGeom tc_geometry(const TreePlan& P, int d, int prec, const TcTile* tile
     G.stage_bytes = G.R_load * 128;
     G.ldD = ((G.N_load + 31) & ~31) + 1;
     const int s_max = std::max(1, std::min(std::min(G.nK, 4), (200 * 1024) / G.stage_bytes));
+    // leaves of at most 256 points: two CTAs per SM, so no more stages than
+    // the selection's shared memory holds anyway (three of 32 KB)
+    const int s_def = P.max_leaf <= 256 ? std::max(1, std::min(s_max, kFastSmem / G.stage_bytes)) : s_max;
     if (tile && tile->S >= 1 && tile->RG >= 32) {
         G.S = std::min(tile->S, s_max);
         G.RG = tile->RG;
     } else {
-        // default: deepest pipeline that fits; rows per epilogue group: 128,
+        // default: deepest pipeline that fits beside a second CTA; rows per epilogue group: 128,
         // 64 or 32 (a divisor of the 128-row block) within 72 KB
-        G.S = s_max;
+        G.S = s_def;
         G.RG = 128;
         while (G.RG > 32 && G.RG * G.ldD * 4 > 72 * 1024) G.RG >>= 1;
     }
     // the pipeline region is reused after the MMAs: by the row-per-thread
     // selection (kFastSmem), by the distance block of the warp-per-row path
-    // and, past both, by the warps' selection scratch
-    G.wsc_off = (std::max(G.RG * G.ldD * 4, 72 * 1024) + 15) & ~15;
+    // and, past it, by the warps' selection scratch (the rescoring of listed
+    // rows reads its columns from the end of kFastSmem: the scratch ends
+    // before them or starts past them)
+    G.wsc_off = (std::max(G.RG * G.ldD * 4, kListBytes - kTcWarps * kLeafWarpScratch) + 15) & ~15;
+    if (G.wsc_off > kListBytes - kTcWarps * kLeafWarpScratch && G.wsc_off < kFastSmem) G.wsc_off = kFastSmem;
     G.pipe_bytes = std::max(std::max(G.S * G.stage_bytes, G.wsc_off + kTcWarps * kLeafWarpScratch), kFastSmem);
     G.pipe_bytes = (G.pipe_bytes + 1023) & ~1023;
-    G.smem = 1024 + G.pipe_bytes + 3 * G.N_load * 4 + 16 + (2 * G.S + 1) * 8 + 16;
+    G.smem = 1024 + G.pipe_bytes + 3 * G.N_load * 4 + 64 + (2 * G.S + 1) * 8 + 16;
     return G;
 }
 
@@ -118,7 +124,7 @@ cudaError_t run_leaf_knn_tc(const XDesc& x, const TreePlan& P, const DevPlan& dp
     if (kp > kTcCand) kp = kTcCand;
     // rows of leaves that are not exact are rescored by the staged kernel
     // (their candidates in [rows][kp] local indices, a flag per leaf)
-    const bool staged = leaf_rescore_staged_ok(x, kp, P.max_leaf);
+    const bool staged = leaf_rescore_staged_ok(kp, P.max_leaf);
     const int nleaves = (int)P.leaf_off.size() - 1;
     uint16_t* cand = staged ? ar.take<uint16_t>((size_t)T * x.n * kp) : nullptr;
     uint8_t* leaf_flag = staged ? ar.take<uint8_t>((size_t)T * nleaves) : nullptr;

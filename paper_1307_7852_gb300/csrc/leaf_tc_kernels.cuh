@@ -258,11 +258,15 @@ __device__ __forceinline__ void reg_bitonic_sort(T (&v)[N])
     }
 }
 
-// Shared memory of the row-per-thread selection (reusing the pipeline):
-// sorted group minima [32][256] u32 (later the halves' sorted runs
-// [2][16][128] u64) and candidate lists [32][256] u64 (later the rows'
-// merged lists [32][128] u64).
-constexpr int kFastSmem = 32 * kTcThreads * 4 + 32 * kTcThreads * 8;
+// Shared memory of the row-per-thread selection (reusing the pipeline): the
+// threads' candidate lists [kListCap][256] of (value, column) pairs -- first
+// the sorted group minima [32][256], later the sorted lists, the halves'
+// sorted runs [2][16][128] u64 of exact leaves -- and the rows' selected
+// columns [128][kListWant] u16.  100 KB: two CTAs per SM beside their tables.
+constexpr int kListCap = 44;   // entries of a thread's list
+constexpr int kListWant = 48;  // largest candidate count of the row-per-thread selection
+constexpr int kListBytes = kListCap * kTcThreads * 8;
+constexpr int kFastSmem = kListBytes + 128 * kListWant * 2;
 
 template <int PREC, int PER, int kDT>
 __global__ void __launch_bounds__(kTcThreads, PER == 16 ? 1 : 2) leaf_tc_kernel(const __grid_constant__ CUtensorMap tmap,
@@ -486,10 +490,16 @@ __global__ void __launch_bounds__(kTcThreads, PER == 16 ? 1 : 2) leaf_tc_kernel(
     // the distances over the columns with the same position in their chunk
     // (32 groups per thread), sorts them; the want-th smallest of the 64
     // minima of a row (both halves) bounds the row's answer.  Pass 2 lists
-    // the columns up to that bound, and the half-0 thread sorts the union of
-    // the row's two lists (at most 32) with a register network.  Rows whose
-    // lists overflow, and all rows when more than 32 candidates are wanted,
-    // take the warp-per-row path below.
+    // the columns up to that bound (about -64 ln(1 - want/64) of them: 24
+    // for 20, 44 for 32, 63 for 40).  A row whose lists hold more than it
+    // wants is cut to the want smallest: its threads sort the listed values,
+    // find the want-th of the two sorted lists and drop what lies above it
+    // (a list longer than the register network: a warp sorts both lists).
+    // Exact leaves then sort the row's union (at most 32) and write the
+    // final lists; the others hand over the selected columns.  Rows whose
+    // lists overflow, rows with equal values at the cut, and all rows when
+    // more than kListWant candidates (32 of an exact leaf) are wanted take
+    // the warp-per-row path below.
     if (!abort_flag) {
         const int quad = w & 3, half = w >> 2;
         const int lr = 32 * quad + lane;
@@ -497,12 +507,14 @@ __global__ void __launch_bounds__(kTcThreads, PER == 16 ? 1 : 2) leaf_tc_kernel(
         const bool row_ok = iloc < m;
         const int kw = exact_leaf ? k : kp;
         const int want = min(kw, m - 1);
-        uint32_t* gsh = reinterpret_cast<uint32_t*>(pipe);                     // [32][256]
-        uint64_t* cand = reinterpret_cast<uint64_t*>(pipe + 32 * kTcThreads * 4);  // [32][256]
+        uint2* list = reinterpret_cast<uint2*>(pipe);       // [kListCap][256]: value bits, column
+        float* fsh = reinterpret_cast<float*>(pipe);        // [32][256]: sorted minima (before the lists)
+        uint16_t* picks = reinterpret_cast<uint16_t*>(pipe + kListBytes);  // [128][kListWant]
         __shared__ int ccount[kTcThreads];
-        __shared__ unsigned char rowflag[128];
+        __shared__ float rowtau[128];
+        __shared__ unsigned char rowflag[128];  // 0 done here, 1 warp-per-row, 2 cut by a warp
         __shared__ int any_overflow;
-        const bool fast = want <= 32;
+        const bool fast = want <= (exact_leaf ? 32 : kListWant);
         if (tid == 0) any_overflow = fast ? 0 : 1;
         if (tid < 128) rowflag[tid] = fast ? 0 : 1;
         __syncthreads();
@@ -517,13 +529,21 @@ __global__ void __launch_bounds__(kTcThreads, PER == 16 ? 1 : 2) leaf_tc_kernel(
         const float kInf = __int_as_float(0x7f800000);
         auto chunk_dv = [&](const uint32_t (&r)[32], int c0, float (&dv)[32]) {
             if (PREC == 1) {
+                // packed pairs: each half rounds like the scalar operations
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
                     const float4 q = *reinterpret_cast<const float4*>(qn + c0 + 4 * i);
-                    const float qv[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-                    for (int e2 = 0; e2 < 4; ++e2)
-                        dv[4 * i + e2] = ni + qv[e2] - 2.f * __uint_as_float(r[4 * i + e2]);
+                    const float2 two = make_float2(-2.f, -2.f), n2 = make_float2(ni, ni);
+                    const float2 lo = __ffma2_rn(
+                        two, make_float2(__uint_as_float(r[4 * i]), __uint_as_float(r[4 * i + 1])),
+                        __fadd2_rn(n2, make_float2(q.x, q.y)));
+                    const float2 hi = __ffma2_rn(
+                        two, make_float2(__uint_as_float(r[4 * i + 2]), __uint_as_float(r[4 * i + 3])),
+                        __fadd2_rn(n2, make_float2(q.z, q.w)));
+                    dv[4 * i] = lo.x;
+                    dv[4 * i + 1] = lo.y;
+                    dv[4 * i + 2] = hi.x;
+                    dv[4 * i + 3] = hi.y;
                 }
             } else {
 #pragma unroll
@@ -584,106 +604,212 @@ __global__ void __launch_bounds__(kTcThreads, PER == 16 ? 1 : 2) leaf_tc_kernel(
 #pragma unroll
                 for (int e = 0; e < 32; ++e) gm[e] = fminf(gm[e], dv[e]);
             });
-            reg_bitonic_sort(gm);
-            float* gshf = reinterpret_cast<float*>(gsh);
+            reg_oddeven_sort(gm);
 #pragma unroll
-            for (int e = 0; e < 32; ++e) gshf[e * kTcThreads + tid] = gm[e];
+            for (int e = 0; e < 32; ++e) fsh[e * kTcThreads + tid] = gm[e];
             __syncthreads();
-            // the want-th smallest of the row's 64 minima (two sorted lists
-            // A, B): binary search for the number i of them taken from A, the
-            // smallest i with A[i] >= B[want - i - 1]
+            // the want-th smallest of two sorted lists of 32 values A (this
+            // thread's) and B (its partner's), value i of thread u at
+            // v[i * stride * 256 + u * stride]: binary search for the number
+            // i of them taken from A, the smallest i with A[i] >= B[want - i - 1]
             const int ptid = tid ^ 128;
-            float tau;
-            {
+            auto want_th = [&](const float* v, int stride) {
                 int lo = max(0, want - 32), hi = min(want, 32);
                 while (lo < hi) {
                     const int i = (lo + hi) >> 1;
-                    const float a = gshf[i * kTcThreads + tid];  // i < hi <= 32
-                    const float b = gshf[(want - i - 1) * kTcThreads + ptid];
+                    const float a = v[(i * kTcThreads + tid) * stride];  // i < hi <= 32
+                    const float b = v[((want - i - 1) * kTcThreads + ptid) * stride];
                     if (a >= b) hi = i;
                     else lo = i + 1;
                 }
-                const float ta = lo > 0 ? gshf[(lo - 1) * kTcThreads + tid] : -kInf;
-                const float tb = want - lo > 0 ? gshf[(want - lo - 1) * kTcThreads + ptid] : -kInf;
-                tau = fmaxf(ta, tb);
-                if (tau == kInf) tau = __int_as_float(0x7f7fffff);  // the invalid columns stay out
-            }
-            // pass 2: the candidates up to the bound
-            int c = 0;
+                const float ta = lo > 0 ? v[((lo - 1) * kTcThreads + tid) * stride] : -kInf;
+                const float tb = want - lo > 0 ? v[((want - lo - 1) * kTcThreads + ptid) * stride] : -kInf;
+                return fmaxf(ta, tb);
+            };
+            float tau = want_th(fsh, 1);
+            if (tau == kInf) tau = __int_as_float(0x7f7fffff);  // the invalid columns stay out
+            __syncthreads();  // the minima are read before the lists replace them
+            // pass 2: the candidates up to the bound; the list's room is
+            // tested every four columns
+            uint32_t at = tc::smem_u32(list + tid);
+            const uint32_t at0 = at;
+            constexpr uint32_t kStep = kTcThreads * 8;
+            bool ovf = false;
             for_chunks([&](const uint32_t (&r)[32], int c0) {
                 float dv[32];
                 chunk_dv(r, c0, dv);
 #pragma unroll
-                for (int e = 0; e < 32; ++e) {
-                    if (dv[e] <= tau) {
-                        if (c < 32) cand[c * kTcThreads + tid] = ((uint64_t)ord_key(dv[e]) << 32) | (uint32_t)(c0 + e);
-                        ++c;
+                for (int e = 0; e < 32; e += 4) {
+                    const bool room = at <= at0 + (kListCap - 4) * kStep;
+                    ovf |= !room;
+                    const float lim = room ? tau : -kInf;
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        if (dv[e + q] <= lim) {
+                            asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(at), "r"(__float_as_uint(dv[e + q])),
+                                         "r"(c0 + e + q)
+                                         : "memory");
+                            at += kStep;
+                        }
                     }
                 }
             });
-            if (c > 32 && row_ok) {
+            int c = (int)((at - at0) / kStep);
+            ccount[tid] = ovf ? 1000 : c;
+            __syncthreads();
+            const int cp = ccount[ptid];
+            // (fewer listed than wanted: distances that are not finite)
+            const bool bad = !row_ok || ovf || cp == 1000 || c + cp < want;
+            if (bad) c = 0;
+            if (row_ok && bad) {
                 rowflag[lr] = 1;
                 any_overflow = 1;
             }
-            ccount[tid] = min(c, 32);
-            __syncthreads();
-            // the union of the row's two lists (slots: list A, then list B),
-            // at most 32 (more overflows): each half sorts 16 slots with a
-            // register network; then the half-0 thread merges the two sorted
-            // runs forward into ranks 0..15 and the half-1 thread backward
-            // into ranks 31..16 (the keys are distinct: no ties to order),
-            // and both write the exact leaves' output (or the list to
-            // rescore)
-            const int rtA = tid & 127, rtB = rtA | 128;  // the row's two threads
-            const int ca = ccount[rtA], cb = ccount[rtB];
-            const bool sel = row_ok && !rowflag[lr] && ca + cb <= 32;
-            uint64_t* srt = reinterpret_cast<uint64_t*>(gsh);  // [2][16][128], minima are dead
-            if (sel) {
-                uint64_t v[16];
+            // rows to cut: more listed than wanted (of an exact leaf: than
+            // its sort takes)
+            const int tot = bad ? 0 : c + cp;
+            const bool cut = !bad && tot > (exact_leaf ? 32 : want);
+            const bool longlist = cut && (c > 32 || cp > 32);
+            if (longlist) rowflag[lr] = 2;
+            const bool cut_warp = __any_sync(KNNG_FULL_MASK, cut);
+            // the listed values, sorted, replace the values in the list (the
+            // columns stay); the originals stay in registers
+            float lv[32];
+            if (cut_warp) {
+                float sv[32];
 #pragma unroll
-                for (int e = 0; e < 16; ++e) {
-                    const int u = 16 * half + e;
-                    v[e] = u < ca ? cand[u * kTcThreads + rtA]
-                                  : (u - ca < cb ? cand[(u - ca) * kTcThreads + rtB] : kKeyMax);
+                for (int e = 0; e < 32; ++e) {
+                    lv[e] = e < c ? __uint_as_float(list[e * kTcThreads + tid].x) : kInf;
+                    sv[e] = lv[e];
                 }
-                reg_bitonic_sort(v);
+                if (__any_sync(KNNG_FULL_MASK, cut && !longlist)) {
+                    reg_oddeven_sort(sv);
+                    if (cut && !longlist) {
 #pragma unroll
-                for (int e = 0; e < 16; ++e) srt[(16 * half + e) * 128 + lr] = v[e];
-            } else if (row_ok && half == 0 && !rowflag[lr]) {
-                rowflag[lr] = 1;
-                any_overflow = 1;
+                        for (int e = 0; e < 32; ++e) list[e * kTcThreads + tid].x = __float_as_uint(sv[e]);
+                    }
+                }
             }
-            __syncthreads();
-            uint64_t* rowlist = reinterpret_cast<uint64_t*>(cand);  // [32][128], the lists are dead
-            if (sel) {
-                const uint64_t* S0 = srt + lr;
-                const uint64_t* S1 = srt + 16 * 128 + lr;
+            const bool any_cut = __syncthreads_or(cut) != 0;
+            if (any_cut) {
+                float t2 = -kInf;
+                if (cut && !longlist) t2 = want_th(reinterpret_cast<const float*>(list), 2);
+                // long lists: one warp per row sorts the values of both
+                // (ordered as unsigned words)
+                if (__syncthreads_or(longlist)) {
+                    for (int rr = w; rr < 128; rr += kTcWarps) {
+                        if (rowflag[rr] != 2) continue;
+                        const int na = ccount[rr], nb = ccount[rr + 128];
+                        uint32_t kv[4];
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            const int u = 32 * e + lane;
+                            kv[e] = u < na ? ord_key(__uint_as_float(list[u * kTcThreads + rr].x))
+                                  : u - na < nb ? ord_key(__uint_as_float(list[(u - na) * kTcThreads + rr + 128].x))
+                                                : 0xFFFFFFFFu;
+                        }
+                        warp_bitonic_sort32<4>(kv);
+                        const int src = (want - 1) >> 2, se = (want - 1) & 3;
+                        uint32_t v = kv[0];
+#pragma unroll
+                        for (int e = 1; e < 4; ++e) v = se == e ? kv[e] : v;
+                        v = __shfl_sync(KNNG_FULL_MASK, v, src);
+                        if (lane == 0) rowtau[rr] = unord_key(v);
+                    }
+                    __syncthreads();
+                    if (longlist) {
+                        t2 = rowtau[lr];
+                        rowflag[lr] = 0;  // both of the row's threads write the same
+                    }
+                }
+                // keep the values up to the cut: the list's columns move up
+                // (with their values for exact leaves, which sort them)
+                if (cut) {
+                    int kept = 0;
+#pragma unroll
+                    for (int e = 0; e < 32; ++e) {
+                        if (e < c && lv[e] <= t2) {
+                            list[kept * kTcThreads + tid] =
+                                make_uint2(__float_as_uint(lv[e]), list[e * kTcThreads + tid].y);
+                            ++kept;
+                        }
+                    }
+                    for (int e = 32; e < c; ++e) {
+                        const uint2 v = list[e * kTcThreads + tid];
+                        if (__uint_as_float(v.x) <= t2) {
+                            list[kept * kTcThreads + tid] = v;
+                            ++kept;
+                        }
+                    }
+                    c = kept;
+                    ccount[tid] = c;
+                }
+                __syncthreads();
+                // equal values at the cut: more kept than wanted, the
+                // warp-per-row path orders them by column
+                if (cut && c + ccount[ptid] != want) {
+                    rowflag[lr] = 1;
+                    any_overflow = 1;
+                }
+                __syncthreads();
+            }
+            const bool sel = row_ok && rowflag[lr] == 0;
+            if (exact_leaf) {
+                // the union of the row's two lists (slots: list A, then list
+                // B), at most 32: each half sorts 16 slots with a register
+                // network; then the half-0 thread merges the two sorted runs
+                // forward into ranks 0..15 and the half-1 thread backward
+                // into ranks 31..16 (the keys are distinct: no ties to
+                // order), and both write the leaf's output
+                const int rtA = tid & 127, rtB = rtA | 128;  // the row's two threads
+                uint64_t* srt = reinterpret_cast<uint64_t*>(pipe);  // [2][16][128], over the lists
                 uint64_t v[16];
-                if (half == 0) {
-                    int i = 0, j = 0;
+                if (sel) {
+                    const int ca = ccount[rtA], cb = ccount[rtB];
 #pragma unroll
                     for (int e = 0; e < 16; ++e) {
-                        const uint64_t a = i < 16 ? S0[i * 128] : kKeyMax;
-                        const uint64_t b = j < 16 ? S1[j * 128] : kKeyMax;
-                        const bool ta = a <= b;
-                        v[e] = ta ? a : b;
-                        i += ta ? 1 : 0;
-                        j += ta ? 0 : 1;
+                        const int u = 16 * half + e;
+                        v[e] = kKeyMax;
+                        if (u < ca + cb) {
+                            const uint2 x = list[u < ca ? u * kTcThreads + rtA : (u - ca) * kTcThreads + rtB];
+                            v[e] = ((uint64_t)ord_key(__uint_as_float(x.x)) << 32) | x.y;
+                        }
                     }
-                } else {
-                    int i = 15, j = 15;
-#pragma unroll
-                    for (int e = 15; e >= 0; --e) {
-                        const uint64_t a = i >= 0 ? S0[i * 128] : 0ull;
-                        const uint64_t b = j >= 0 ? S1[j * 128] : 0ull;
-                        const bool ta = a > b;
-                        v[e] = ta ? a : b;
-                        i -= ta ? 1 : 0;
-                        j -= ta ? 0 : 1;
-                    }
+                    reg_bitonic_sort(v);
                 }
-                const int r0s = 16 * half;  // rank of v[0]
-                if (exact_leaf) {
+                __syncthreads();  // the lists are read before the runs replace them
+                if (sel) {
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) srt[(16 * half + e) * 128 + lr] = v[e];
+                }
+                __syncthreads();
+                if (sel) {
+                    const uint64_t* S0 = srt + lr;
+                    const uint64_t* S1 = srt + 16 * 128 + lr;
+                    if (half == 0) {
+                        int i = 0, j = 0;
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) {
+                            const uint64_t a = i < 16 ? S0[i * 128] : kKeyMax;
+                            const uint64_t b = j < 16 ? S1[j * 128] : kKeyMax;
+                            const bool ta = a <= b;
+                            v[e] = ta ? a : b;
+                            i += ta ? 1 : 0;
+                            j += ta ? 0 : 1;
+                        }
+                    } else {
+                        int i = 15, j = 15;
+#pragma unroll
+                        for (int e = 15; e >= 0; --e) {
+                            const uint64_t a = i >= 0 ? S0[i * 128] : 0ull;
+                            const uint64_t b = j >= 0 ? S1[j * 128] : 0ull;
+                            const bool ta = a > b;
+                            v[e] = ta ? a : b;
+                            i -= ta ? 1 : 0;
+                            j -= ta ? 0 : 1;
+                        }
+                    }
+                    const int r0s = 16 * half;  // rank of v[0]
                     const int gi = lid[iloc];
                     int32_t* oi = out_ids + ((int64_t)t * n + gi) * k;
                     float* od = out_d + ((int64_t)t * n + gi) * k;
@@ -719,42 +845,42 @@ __global__ void __launch_bounds__(kTcThreads, PER == 16 ? 1 : 2) leaf_tc_kernel(
                             oi[s2] = -1;
                             od[s2] = __int_as_float(0x7f800000);
                         }
-                } else if (to_cands) {
-                    uint16_t* oc = cand_out + (rowbase + iloc) * kp;
-                    if ((kp & 3) == 0 && want == kp) {
-                        // four local indices a store (row starts 8-byte aligned)
-#pragma unroll
-                        for (int e = 0; e < 16; e += 4)
-                            if (r0s + e < want) {
-                                uint2 u;
-                                u.x = ((uint32_t)v[e] & 0xFFFFu) | ((uint32_t)v[e + 1] << 16);
-                                u.y = ((uint32_t)v[e + 2] & 0xFFFFu) | ((uint32_t)v[e + 3] << 16);
-                                *reinterpret_cast<uint2*>(oc + r0s + e) = u;
-                            }
+                }
+                __syncthreads();
+            } else {
+                // the row's columns (their order does not matter): half 0
+                // from the front, half 1 up to the end
+                const int stride = to_cands ? kp : kListWant;
+                if (sel) {
+                    uint16_t* o = picks + lr * stride + (half ? want - c : 0);
+                    for (int e = 0; e < c; ++e) o[e] = (uint16_t)list[e * kTcThreads + tid].y;
+                }
+                __syncthreads();
+                if (to_cands) {
+                    // the block's rows are contiguous in the output; rows of
+                    // the warp-per-row path are written again below
+                    const int cnt = min(128, m - r0) * kp;
+                    uint16_t* oc = cand_out + (rowbase + r0) * kp;
+                    if ((kp & 1) == 0) {
+                        for (int e = tid; e < cnt / 2; e += kTcThreads)
+                            reinterpret_cast<uint32_t*>(oc)[e] = reinterpret_cast<const uint32_t*>(picks)[e];
                     } else {
-#pragma unroll
-                        for (int e = 0; e < 16; ++e)
-                            if (r0s + e < want) oc[r0s + e] = (uint16_t)(uint32_t)v[e];
+                        for (int e = tid; e < cnt; e += kTcThreads) oc[e] = picks[e];
                     }
                 } else {
-#pragma unroll
-                    for (int e = 0; e < 16; ++e)
-                        if (r0s + e < want) rowlist[(r0s + e) * 128 + lr] = v[e];
+                    // rescore the listed candidates of each row, one warp per row
+                    for (int rr = w; rr < 128; rr += kTcWarps) {
+                        const int il2 = r0 + rr;
+                        if (il2 >= m) break;
+                        if (rowflag[rr]) continue;
+                        const int gi = lid[il2];
+                        leaf_rescore_list(L, lid, il2, picks + rr * stride, want, k,
+                                          wsc + (size_t)kLeafWarpScratch * w, out_ids + ((int64_t)t * n + gi) * k,
+                                          out_d + ((int64_t)t * n + gi) * k);
+                    }
                 }
+                __syncthreads();
             }
-            __syncthreads();
-            if (!exact_leaf && !to_cands) {
-                // rescore the listed candidates of each row, one warp per row
-                for (int rr = w; rr < 128; rr += kTcWarps) {
-                    const int il2 = r0 + rr;
-                    if (il2 >= m) break;
-                    if (rowflag[rr]) continue;
-                    const int gi = lid[il2];
-                    leaf_rescore_list(L, lid, il2, rowlist + rr, 128, want, k, wsc + (size_t)kLeafWarpScratch * w,
-                                      out_ids + ((int64_t)t * n + gi) * k, out_d + ((int64_t)t * n + gi) * k);
-                }
-            }
-            __syncthreads();
         }
         if (any_overflow) {
             // warp-per-row path for the rows not done above
