@@ -10,22 +10,22 @@
 // rows stream through shared memory instead, in 32-entry slices (one block
 // of the canonical distance), double-buffered, so each row of the leaf
 // crosses L2 once per tree:
-//   * one thread per row holds its own slice in registers and one running
-//     sum per candidate; per slice it forms the eight 4-entry partials of
-//     every candidate pair, closes the block by the butterfly and adds it to
-//     the pair's sum -- exactly the canonical distance, block by block;
+//   * one thread per row holds its own slice in registers; per slice it
+//     forms the eight 4-entry partials of every candidate pair, closes the
+//     block by the butterfly and adds it to the pair's running sum in shared
+//     memory -- exactly the canonical distance, block by block;
 //   * thread r reads the slice's eight 16-byte columns in the order
 //     u ^ (r mod 8), so the eight threads of a quarter warp touch eight
 //     different bank groups whatever rows they read;
 //   * at the end every row sorts its candidates by (distance, id) and keeps
 //     the k best.
 // What bounds it: shared-memory bandwidth, 128 bytes a pair and slice (four
-// wavefronts per 16-byte load of a warp), so a pair listed by both of its
-// rows is scored by one of them only, and each thread's own pairs come first
-// in its list: a warp's loop ends at its longest list of own pairs.
-// 16-byte aligned FP32 rows are copied by cp.async; other rows (FP16, bytes,
-// unaligned) are loaded a slice ahead into registers and widened on the way
-// to shared memory.
+// wavefronts per 16-byte load of a warp; the running sum adds two).  So a
+// pair listed by both of its rows is scored by one of them only, the threads
+// take the rows in order of their number of pairs (a warp's loop ends at its
+// longest list), and the next pair's slice is loaded while one is summed.
+// 16-byte aligned FP32 rows are copied by cp.async a slice ahead; other rows
+// (FP16, bytes, unaligned) are loaded, widened and stored.
 // Leaves that are exact in reduced precision (their lists are final) are
 // skipped by a flag the leaf kernel writes.
 #include <algorithm>
@@ -41,21 +41,20 @@ constexpr int kSlice = 32;       // floats per row and slice (one block of the d
 constexpr int kMaxCand = 40;     // candidates per row handled here
 }  // namespace
 
-// Canonical block value of a pair: own slice a (columns in the order
-// u ^ x, u = 0..7, already in registers), candidate slice b in shared
-// memory.  s[u] is the partial of column u ^ x; since the block's butterfly
+// Canonical block value of a pair: own slice a and candidate slice b, columns
+// in the order u ^ x, u = 0..7.  s[u] is the partial of column u ^ x; since the block's butterfly
 // pairs columns by xor (q with q ^ 4, then q ^ 2, then q ^ 1), relabelling
 // them by xor with x only swaps the operands of some additions, so the tree
 // below over s[] gives the block value bit for bit -- and, t = a - b and
 // b - a squaring alike, the same value whichever row is the own one.
 // (Scalar FP32: packed pairs need their operands in adjacent registers,
 // which these columns are not, and measured slower.)
-__device__ __forceinline__ float slice_block(const float4 (&a)[8], const float4* __restrict__ b, int x)
+__device__ __forceinline__ float slice_block(const float4 (&a)[8], const float4 (&b)[8])
 {
     float s[8];
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-        const float4 v = b[u ^ x];
+        const float4 v = b[u];
         float acc = 0.f, t;
         t = a[u].x - v.x; acc = fmaf(t, t, acc);
         t = a[u].y - v.y; acc = fmaf(t, t, acc);
@@ -69,8 +68,9 @@ __device__ __forceinline__ float slice_block(const float4 (&a)[8], const float4*
 // grid (nleaves, T); blockDim >= the largest leaf (multiple of 32, <= 512).
 // cand: [T * n][kp] local indices (u16) of every row's candidates, the first
 // want = min(kp, m - 1) valid, kp <= KC.  kAsync: FP32 rows, 16-byte aligned,
-// ld % 4 == 0.  nbuf: slices in shared memory, 2 or (kAsync) 3 -- with three
-// a slice needs one barrier instead of two.
+// ld % 4 == 0.  nbuf: slices in shared memory; with 2 the next one is loaded
+// while one is scored, with 1 between two of them, with 3 (kAsync) a slice
+// needs one barrier instead of two.
 //
 // A pair listed by both of its rows (r in c's list and c in r's) is scored
 // once: the canonical distance is symmetric bit for bit, so the other row
@@ -84,6 +84,17 @@ __device__ __forceinline__ float slice_block(const float4 (&a)[8], const float4*
 constexpr int kBitRow = 21;      // words of a row's bitmap (16) and prefix counts (4); odd: no bank conflicts
 constexpr int kNoSlot = 63;
 
+// Bytes of the slices (and, over them, the bitmaps and the table).
+__host__ __device__ constexpr size_t slice_bytes(int mp, int kp, int nbuf)
+{
+    const size_t sl = (size_t)nbuf * 8 * sizeof(float4), tb = (size_t)kp * sizeof(float);
+    return (size_t)mp * (sl > tb ? sl : tb);
+}
+
+// Up to 24 pairs a row keep their running sums in registers (the pair loop
+// unrolled); more keep them in shared memory (rolled).
+__host__ __device__ constexpr bool regs_hold(int kc) { return kc <= 24; }
+
 template <int KC, int kDT, bool kAsync>
 __global__ void __launch_bounds__(512, 1) leaf_rescore_staged_kernel(
     RowLoader<kDT> L, int64_t n, const int32_t* __restrict__ perm,
@@ -91,17 +102,21 @@ __global__ void __launch_bounds__(512, 1) leaf_rescore_staged_kernel(
     const uint16_t* __restrict__ cand, int kp, uint32_t kp_magic, int nbuf, int k, int32_t* __restrict__ out_ids,
     float* __restrict__ out_d)
 {
+    constexpr bool kRegs = regs_hold(KC);
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ int hist[64];
     const int t = blockIdx.y, leaf = blockIdx.x;
     if (leaf_exact && leaf_exact[(int64_t)t * nleaves + leaf]) return;
     const int off = leaf_off[leaf];
     const int m = leaf_off[leaf + 1] - off;
     const int mp = (m + 7) & ~7;
     const int d = L.d;
-    // [nbuf][mp][8] float4 slices | lid[mp] | list[kp][mp] u16
+    // [nbuf][mp][8] float4 slices | lid[mp] | tot[kp][mp] f32 (!kRegs) | list[kp][mp] u16 | order[mp] u16
     float4* buf = reinterpret_cast<float4*>(smem_raw);
-    int32_t* lid = reinterpret_cast<int32_t*>(buf + (size_t)nbuf * mp * 8);
-    uint16_t* list = reinterpret_cast<uint16_t*>(lid + mp);
+    int32_t* lid = reinterpret_cast<int32_t*>(smem_raw + slice_bytes(mp, kp, nbuf));
+    float* tot = reinterpret_cast<float*>(lid + mp);
+    uint16_t* list = reinterpret_cast<uint16_t*>(tot + (kRegs ? 0 : (size_t)kp * mp));
+    uint16_t* order = list + (size_t)kp * mp;
     // over the slices: bits[mp][kBitRow] before them, res[kp][mp] after
     uint32_t* bits = reinterpret_cast<uint32_t*>(buf);
     float* res = reinterpret_cast<float*>(buf);
@@ -112,15 +127,37 @@ __global__ void __launch_bounds__(512, 1) leaf_rescore_staged_kernel(
     const bool active = tid < m;
     const int want = min(kp, m - 1);
     for (int e = tid; e < mp * kBitRow; e += blockDim.x) bits[e] = 0u;
+    for (int e = tid; e < 64; e += blockDim.x) hist[e] = 0;  // (a block may have 32 threads)
     __syncthreads();
-    // the leaf's candidates are contiguous; entry e is candidate e mod kp of
-    // row e / kp (kp_magic = 2^32 / kp rounded up: exact below 2^16)
-    const uint16_t* cleaf = cand + rowbase * kp;
-    for (int e = tid; e < m * kp; e += blockDim.x) {
-        const int r = kp == 1 ? e : (int)__umulhi((uint32_t)e, kp_magic);
-        if (e - r * kp < want) {
-            const int c = cleaf[e];
-            atomicOr(&bits[r * kBitRow + (c >> 5)], 1u << (c & 31));
+    // the leaf's candidates are contiguous, read as aligned groups of eight;
+    // entry e is candidate e mod kp of row e / kp (kp_magic = 2^32 / kp
+    // rounded up: exact below 2^16)
+    {
+        const int64_t first = rowbase * kp;
+        const int lead = (int)(first & 7);
+        const uint4* src = reinterpret_cast<const uint4*>(cand + (first - lead));
+        const int groups = (m * kp + lead + 7) >> 3;
+        for (int g0 = tid; g0 < groups; g0 += 4 * blockDim.x) {
+            uint4 v[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int g = g0 + q * blockDim.x;
+                v[q] = g < groups ? src[g] : make_uint4(0u, 0u, 0u, 0u);
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const uint32_t wv[4] = {v[q].x, v[q].y, v[q].z, v[q].w};
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const int e = 8 * (g0 + q * (int)blockDim.x) + j - lead;
+                    if (e < 0 || e >= m * kp) continue;
+                    const int r = kp == 1 ? e : (int)__umulhi((uint32_t)e, kp_magic);
+                    if (e - r * kp < want) {
+                        const uint32_t c = (wv[j >> 1] >> (16 * (j & 1))) & 0xFFFFu;
+                        if (c < (uint32_t)m) atomicOr(&bits[r * kBitRow + (c >> 5)], 1u << (c & 31u));
+                    }
+                }
+            }
         }
     }
     __syncthreads();
@@ -137,124 +174,165 @@ __global__ void __launch_bounds__(512, 1) leaf_rescore_staged_kernel(
         }
     }
     __syncthreads();
-    // the row's list, an entry being candidate | slot << 9: the pairs it
+    // row tid's list, an entry being candidate | slot << 9: the pairs it
     // scores from the front, with the slot in the candidate's table row
     // (kNoSlot: the candidate does not list this row), the others from the
     // end, with the slot in the own table row
-    int nown = 0;
+    int mine = 0;
     if (active) {
-        int back = want, rank = 0;
+        int back = want, z = 0;
         const int myw = tid >> 5;
-        for (int z = 0; z < 16 && rank < want; ++z) {
-            uint32_t word = bits[tid * kBitRow + z];
-            while (word) {
-                const int c = 32 * z + __ffs((int)word) - 1;
-                word &= word - 1u;
-                const uint32_t cw = bits[c * kBitRow + myw];
-                const bool listed = (cw >> lane) & 1u;
-                if (!listed || ((c > tid) == (((c + tid) & 1) != 0))) {
-                    const uint32_t pre = (bits[c * kBitRow + 16 + (myw >> 2)] >> (8 * (myw & 3))) & 0xFFu;
-                    const int slot = listed ? (int)pre + __popc(cw & lanemask_lt()) : kNoSlot;
-                    list[nown * mp + tid] = (uint16_t)(c | (slot << 9));
-                    ++nown;
-                } else {
-                    --back;
-                    list[back * mp + tid] = (uint16_t)(c | (rank << 9));
-                }
-                ++rank;
+        uint32_t word = bits[tid * kBitRow];
+        for (int rank = 0; rank < want; ++rank) {
+            while (word == 0u && z < 15) word = bits[tid * kBitRow + ++z];
+            if (word == 0u) break;
+            const int c = 32 * z + __ffs((int)word) - 1;
+            word &= word - 1u;
+            const uint32_t cw = bits[c * kBitRow + myw];
+            const bool listed = (cw >> lane) & 1u;
+            if (!listed || ((c > tid) == (((c + tid) & 1) != 0))) {
+                const uint32_t pre = (bits[c * kBitRow + 16 + (myw >> 2)] >> (8 * (myw & 3))) & 0xFFu;
+                const int slot = listed ? (int)pre + __popc(cw & lanemask_lt()) : kNoSlot;
+                list[mine * mp + tid] = (uint16_t)(c | (slot << 9));
+                ++mine;
+            } else {
+                --back;
+                list[back * mp + tid] = (uint16_t)(c | (rank << 9));
             }
         }
+        // (a leaf whose candidate kernel gave up lists fewer)
+        for (int i = mine; i < back; ++i) list[i * mp + tid] = (uint16_t)tid;
+        atomicAdd(&hist[mine], 1);
     }
-    const int wmax = __reduce_max_sync(KNNG_FULL_MASK, nown);
     __syncthreads();  // the bitmaps are read before the slices replace them
 
     const int nslices = (d + kSlice - 1) / kSlice;
-    // slice sl into buffer b: cp.async, or loads a slice ahead (fetch) that
-    // put() widens into the buffer; thread u copies columns u, u + blockDim, ...
+    // slice sl into buffer b
     auto stage = [&](int sl, int b) {
         float4* dst = buf + (size_t)b * mp * 8;
-        for (int u = tid; u < m * 8; u += blockDim.x) {
-            const int r = u >> 3, col = u & 7;
-            const int j = sl * kSlice + 4 * col;
-            const int avail = d - j;
-            const float* src = static_cast<const float*>(L.X) + L.row_off(lid[r]);
-            const int bytes = avail >= 4 ? 16 : (avail > 0 ? 4 * avail : 0);
-            cp_async16(dst + (size_t)r * 8 + col, bytes > 0 ? src + j : src, bytes);
-        }
-        cp_async_commit();
-    };
-    float4 pf[kAsync ? 1 : 8];
-    auto fetch = [&](int sl) {
+        if constexpr (kAsync) {
+            // (blockDim is a multiple of 8: a thread copies one column)
+            const int j = sl * kSlice + 4 * (tid & 7);
+            const int bytes = min(max(4 * (d - j), 0), 16);
+            const float* base = static_cast<const float*>(L.X) + (bytes > 0 ? j : 0);
+            for (int u = tid; u < m * 8; u += blockDim.x)
+                cp_async16(dst + u, base + L.row_off(lid[u >> 3]), bytes);
+            cp_async_commit();
+        } else {
+            // eight columns a thread at most (blockDim >= m), four loads in flight
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int u = tid + i * blockDim.x;
-            const int j = sl * kSlice + 4 * (u & 7);
-            pf[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (u < m * 8 && j < d) pf[i] = L.load4(lid[u >> 3], j);
+            for (int i0 = 0; i0 < 8; i0 += 4) {
+                float4 v[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int u = tid + (i0 + i) * blockDim.x;
+                    const int j = sl * kSlice + 4 * (u & 7);
+                    v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (u < m * 8 && j < d) v[i] = L.load4(lid[u >> 3], j);
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int u = tid + (i0 + i) * blockDim.x;
+                    if (u < m * 8) dst[u] = v[i];
+                }
+            }
         }
     };
-    auto put = [&](int b) {
-        float4* dst = buf + (size_t)b * mp * 8;
+    stage(0, 0);
+    // the rows in order of their number of pairs (a counting sort, longest
+    // first; the order of equal ones does not matter)
+    if (tid < 32) {
+        const int a = hist[63 - 2 * tid], b2 = hist[62 - 2 * tid];
+        int incl = a + b2;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int u = tid + i * blockDim.x;
-            if (u < m * 8) dst[u] = pf[i];
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(KNNG_FULL_MASK, incl, o);
+            if (lane >= o) incl += v;
         }
-    };
-    const int x8 = tid & 7;  // columns read in the order u ^ x8: a quarter warp hits eight bank groups
-
-    float tot[KC];
-#pragma unroll
-    for (int i = 0; i < KC; ++i) tot[i] = 0.f;
-    if constexpr (kAsync) {
-        stage(0, 0);
-        if (nbuf == 3 && nslices > 1) stage(1, 1);
-    } else {
-        fetch(0);
-        put(0);
+        __syncwarp();
+        hist[63 - 2 * tid] = incl - a - b2;
+        hist[62 - 2 * tid] = incl - b2;
     }
+    __syncthreads();
+    if (active) order[atomicAdd(&hist[mine], 1)] = (uint16_t)(tid | (mine << 9));
+    __syncthreads();
+    const int row = active ? order[tid] & 511 : 0;
+    const int nown = active ? order[tid] >> 9 : 0;
+    const int wmax = __reduce_max_sync(KNNG_FULL_MASK, nown);
+    const int x8 = tid & 7;  // columns read in the order u ^ x8: a quarter warp hits eight bank groups
+    auto load_slice = [&](float4 (&v)[8], const float4* __restrict__ b) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = b[u ^ x8];
+    };
+    // pair i's candidate (past the own pairs: the row itself, whose sum is
+    // not kept)
+    auto cand_of = [&](int i) { return i < nown ? list[i * mp + row] & 511 : row; };
+    float sum[kRegs ? KC : 1];
+    if constexpr (kRegs) {
+#pragma unroll
+        for (int i = 0; i < KC; ++i) sum[i] = 0.f;
+    } else {
+        for (int i = 0; i < wmax; ++i) tot[i * mp + (active ? tid : 0)] = 0.f;
+    }
+    if (nbuf == 3 && nslices > 1) stage(1, 1);
     int bsl = 0;  // buffer of slice sl
     for (int sl = 0; sl < nslices; ++sl) {
+        const bool ahead = nbuf >= 2 && sl + 1 < nslices;
+        if (nbuf == 2 && ahead) stage(sl + 1, bsl ^ 1);
         if constexpr (kAsync) {
-            if (nbuf == 2 && sl + 1 < nslices) stage(sl + 1, bsl ^ 1);
-            if (sl + 1 < nslices) cp_async_wait<1>();
+            if (ahead) cp_async_wait<1>();
             else cp_async_wait<0>();
-        } else {
-            if (sl + 1 < nslices) fetch(sl + 1);
         }
         __syncthreads();
         // (three buffers: the one of slice sl - 1, whose readers passed the
         // barrier)
-        if (kAsync && nbuf == 3 && sl + 2 < nslices) stage(sl + 2, bsl == 0 ? 2 : bsl - 1);
+        if (nbuf == 3 && sl + 2 < nslices) stage(sl + 2, bsl == 0 ? 2 : bsl - 1);
         if (wmax > 0) {
             const float4* B = buf + (size_t)bsl * mp * 8;
             float4 a[8];
-            const int self = active ? tid : 0;
+            load_slice(a, B + (size_t)row * 8);
+            if constexpr (kRegs) {
 #pragma unroll
-            for (int u = 0; u < 8; ++u) a[u] = B[(size_t)self * 8 + (u ^ x8)];
-#pragma unroll
-            for (int i = 0; i < KC; ++i) {
-                if (i >= wmax) break;  // uniform over the warp
-                const int c = i < nown ? list[i * mp + tid] & 511 : self;
-                tot[i] = tot[i] + slice_block(a, B + (size_t)c * 8, x8);
+                for (int i = 0; i < KC; ++i) {
+                    if (i >= wmax) break;  // uniform over the warp
+                    float4 v[8];
+                    load_slice(v, B + (size_t)cand_of(i) * 8);
+                    sum[i] = sum[i] + slice_block(a, v);
+                }
+            } else {
+                float4 v0[8], v1[8];
+                load_slice(v0, B + (size_t)cand_of(0) * 8);
+                int c1 = cand_of(1);
+                float* tp = tot + (active ? tid : 0);
+                for (int i = 0; i < wmax; i += 2) {
+                    load_slice(v1, B + (size_t)c1 * 8);
+                    const int c2 = cand_of(i + 2), c3 = cand_of(i + 3);
+                    const float s0 = tp[i * mp] + slice_block(a, v0);
+                    if (i < nown) tp[i * mp] = s0;
+                    load_slice(v0, B + (size_t)c2 * 8);
+                    if (i + 1 < nown) tp[(i + 1) * mp] = tp[(i + 1) * mp] + slice_block(a, v1);
+                    c1 = c3;
+                }
             }
         }
-        if constexpr (!kAsync) {
-            if (sl + 1 < nslices) put(bsl ^ 1);  // its last readers passed the barrier above
-        } else if (nbuf == 2) {
-            __syncthreads();  // the buffer of this slice is staged again two slices on
-        }
+        if (nbuf < 3) __syncthreads();  // the buffer of this slice is staged again
+        if (nbuf == 1 && sl + 1 < nslices) stage(sl + 1, 0);
         bsl = bsl + 1 == nbuf ? 0 : bsl + 1;
     }
     __syncthreads();
     // exchange: the pairs another row is to take go to its slot
-    if (active) {
+    if constexpr (kRegs) {
 #pragma unroll
         for (int i = 0; i < KC; ++i)
             if (i < nown) {
-                const int e = list[i * mp + tid];
-                if ((e >> 9) != kNoSlot) res[(e >> 9) * mp + (e & 511)] = tot[i];
+                const int e = list[i * mp + row];
+                if ((e >> 9) != kNoSlot) res[(e >> 9) * mp + (e & 511)] = sum[i];
             }
+    } else {
+        for (int i = 0; i < nown; ++i) {
+            const int e = list[i * mp + row];
+            if ((e >> 9) != kNoSlot) res[(e >> 9) * mp + (e & 511)] = tot[i * mp + tid];
+        }
     }
     __syncthreads();
     if (!active) return;
@@ -263,14 +341,16 @@ __global__ void __launch_bounds__(512, 1) leaf_rescore_staged_kernel(
     for (int i = 0; i < KC; ++i) {
         key[i] = kKeyMax;
         if (i < want) {
-            const int e = list[i * mp + tid];
-            const float dist = i < nown ? tot[i] : res[(e >> 9) * mp + tid];
+            const int e = list[i * mp + row];
+            float dist = kRegs ? sum[kRegs ? i : 0] : 0.f;
+            if (i >= nown) dist = res[(e >> 9) * mp + row];
+            else if (!kRegs) dist = tot[i * mp + tid];
             key[i] = pack_key(dist, (uint32_t)lid[e & 511]);
         }
     }
     // the k best of the row's candidates by (distance, point id)
     reg_oddeven_sort(key);
-    const int gi = lid[tid];
+    const int gi = lid[row];
     int32_t* oi = out_ids + ((int64_t)t * n + gi) * k;
     float* od = out_d + ((int64_t)t * n + gi) * k;
     const float kInf = __int_as_float(0x7f800000);
@@ -302,16 +382,17 @@ __global__ void __launch_bounds__(512, 1) leaf_rescore_staged_kernel(
     }
 }
 
-static size_t staged_smem(int max_leaf, int kp, int nbuf)
+static size_t staged_smem(int max_leaf, int kp, int nbuf, bool regs)
 {
     const size_t mp = (size_t)((max_leaf + 7) & ~7);
-    return std::max(nbuf * mp * 8 * sizeof(float4), mp * kBitRow * sizeof(uint32_t)) + mp * sizeof(int32_t) +
-           mp * kp * sizeof(uint16_t);
+    static_assert(8 * sizeof(float4) >= kBitRow * sizeof(uint32_t), "the bitmaps fit one slice");
+    return slice_bytes((int)mp, kp, nbuf) + mp * (sizeof(int32_t) + sizeof(uint16_t)) +
+           mp * kp * ((regs ? 0 : sizeof(float)) + sizeof(uint16_t));
 }
 
 bool leaf_rescore_staged_ok(int kp, int max_leaf)
 {
-    return kp <= kMaxCand && max_leaf <= 512 && staged_smem(max_leaf, kp, 2) <= 220 * 1024;
+    return kp <= kMaxCand && max_leaf <= 512 && staged_smem(max_leaf, kp, 1, false) <= 226 * 1024;
 }
 
 template <int KC, int kDT, bool kAsync>
@@ -321,10 +402,13 @@ static cudaError_t launch_staged(const XDesc& x, const TreePlan& P, const DevPla
 {
     const int nleaves = (int)P.leaf_off.size() - 1;
     const int threads = std::max(32, (P.max_leaf + 31) & ~31);
-    // a third slice where it costs no resident CTA: more than 256 threads
-    // leave registers for one CTA per SM anyway
-    const int nbuf = kAsync && threads > 256 && staged_smem(P.max_leaf, kp, 3) <= 220 * 1024 ? 3 : 2;
-    const size_t smem = staged_smem(P.max_leaf, kp, nbuf);
+    // as many slices as there is room for, with at most 256 threads beside
+    // the second CTA that the registers allow
+    constexpr bool regs = regs_hold(KC);
+    const size_t room = (threads <= 256 ? 112 : 226) * (size_t)1024;
+    int nbuf = kAsync ? 3 : 2;
+    while (nbuf > 1 && staged_smem(P.max_leaf, kp, nbuf, regs) > room) --nbuf;
+    const size_t smem = staged_smem(P.max_leaf, kp, nbuf, regs);
     const uint32_t kp_magic = (uint32_t)((((uint64_t)1 << 32) + kp - 1) / kp);
     auto kern = leaf_rescore_staged_kernel<KC, kDT, kAsync>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
