@@ -411,7 +411,13 @@ int knng_normalize_rows(knng_handle* h, const void* X, int32_t dtype, int64_t n,
 /* Exact k-NN lists (Def. 1) of nq query points against all n points, by
  * brute force with the same FP32 distance as the graph (the yardstick of the
  * accuracy measure of Sec. 4).  queries: device int32 [nq] point ids;
- * ids, dists: device [nq][k], ordered by (distance, id). */
+ * ids, dists: device [nq][k], ordered by (distance, id).
+ * From 2,048 points on, pairs that cannot be listed are ruled out by a
+ * tensor-core pass with a proven bound first (same lists); its scratch -- a
+ * bfloat16 copy of X and up to 64 MB -- is kept by the handle, and the calls
+ * of one handle on several streams are ordered by an event.  A call on a
+ * stream that is being captured, or without memory for the scratch, takes
+ * the direct form. */
 int knng_exact_knn(knng_handle* h, const void* X, int32_t dtype, int64_t n, int32_t d, int64_t ld,
                    const int32_t* queries, int64_t nq, int32_t k, int32_t* ids, float* dists,
                    void* stream);

@@ -70,6 +70,12 @@ struct knng_handle {
     std::vector<float> div_rates;  // their effective rates r_m (adaptive builds)
     char* staging = nullptr;     // device copies of knng_build_host's buffers (grow-only)
     size_t staging_size = 0;
+    // scratch of knng_exact_knn, apart from ws: its calls may run on another
+    // stream than the handle's other work, and the event orders them among
+    // themselves
+    char* exact_ws = nullptr;
+    size_t exact_ws_size = 0;
+    cudaEvent_t exact_done = nullptr;
     long long wait_cycles = 0;   // limit of the leaf kernel's pipeline waits (0: about 1 s)
     unsigned long long* prop_stats = nullptr;  // caller's read counters, 2 per round
     int prop_stats_rounds = 0;
@@ -174,6 +180,45 @@ int ensure_plan(knng_handle* h, int64_t n, int g, cudaStream_t st)
     h->dplan.chunks = reinterpret_cast<const Chunk*>(h->plan_dev + o_c);
     h->dplan.leaf_off = reinterpret_cast<const int32_t*>(h->plan_dev + o_l);
     return KNNG_OK;
+}
+
+// Scratch of the filtered exact k-NN on st, after its last user's work.
+// False when it cannot be had -- no memory, or st is being captured (a
+// recorded graph may outlive the scratch): the caller then takes the form
+// that needs none.
+bool exact_scratch(knng_handle* h, const XDesc& x, int nq, int k, cudaStream_t st)
+{
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return false;
+    }
+    if (!h->exact_done && cudaEventCreateWithFlags(&h->exact_done, cudaEventDisableTiming) != cudaSuccess) {
+        cudaGetLastError();
+        h->exact_done = nullptr;
+        return false;
+    }
+    if (h->exact_ws && cudaStreamWaitEvent(st, h->exact_done, 0) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    Arena m;
+    run_exact_knn_tc(x, nullptr, nq, k, nullptr, nullptr, nullptr, m, st);
+    if (m.off <= h->exact_ws_size) return true;
+    if (h->exact_ws) {
+        cudaFreeAsync(h->exact_ws, st);
+        h->exact_ws = nullptr;
+        h->exact_ws_size = 0;
+    }
+    const size_t want = m.off + (m.off >> 3) + (1 << 20);
+    void* p = nullptr;
+    if (cudaMallocAsync(&p, want, st) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    h->exact_ws = static_cast<char*>(p);
+    h->exact_ws_size = want;
+    return true;
 }
 
 size_t dtype_size(int32_t dtype)
@@ -503,6 +548,8 @@ int knng_destroy(knng_handle* h)
         if (h->plan_dev) cudaFree(h->plan_dev);
         if (h->dev_err) cudaFree(h->dev_err);
         if (h->staging) cudaFree(h->staging);
+        if (h->exact_ws) cudaFree(h->exact_ws);
+        if (h->exact_done) cudaEventDestroy(h->exact_done);
         BatchCache& B = h->batch;
         if (B.exec) cudaGraphExecDestroy(B.exec);
         if (B.graph) cudaGraphDestroy(B.graph);
@@ -815,7 +862,17 @@ int knng_exact_knn(knng_handle* h, const void* X, int32_t dtype, int64_t n, int3
     if (!queries || !ids || !dists) return fail(h, KNNG_ERR_INVALID_ARG, "NULL pointer");
     if (d > 2048) return fail(h, KNNG_ERR_UNSUPPORTED, "exact k-NN supports d <= 2048");
     DeviceGuard dg(h->device);
-    cudaError_t e = run_exact_knn(x, queries, (int)nq, k, ids, dists, static_cast<cudaStream_t>(stream));
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    cudaError_t e;
+    if (exact_tc_ok(x, (int)nq) && exact_scratch(h, x, (int)nq, k, st)) {
+        Arena a;
+        a.base = h->exact_ws;
+        e = run_exact_knn_tc(x, queries, (int)nq, k, ids, dists, h->dev_err, a, st);
+        const cudaError_t e2 = cudaEventRecord(h->exact_done, st);
+        if (e == cudaSuccess) e = e2;
+    } else {
+        e = run_exact_knn(x, queries, (int)nq, k, ids, dists, st);
+    }
     if (e != cudaSuccess) return cuda_fail(h, e, "exact k-NN");
     return KNNG_OK;
 }

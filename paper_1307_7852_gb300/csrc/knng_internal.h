@@ -259,8 +259,13 @@ cudaError_t run_propagate_pairwise(const XDesc& x, int k, const int32_t* order, 
                                    const float* d_in, const unsigned long long* flags_in, int32_t* ids, float* dists,
                                    unsigned long long* flags_out, const PairScratch& s, int* err, cudaStream_t st);
 
+// need (nullable): answer only the queries marked there.
 cudaError_t run_exact_knn(const XDesc& x, const int32_t* queries, int nq, int k, int32_t* ids,
-                          float* dists, cudaStream_t st);
+                          float* dists, cudaStream_t st, const uint8_t* need = nullptr);
+// The same lists with the pairs filtered on the tensor cores (exact.cu).
+bool exact_tc_ok(const XDesc& x, int nq);
+cudaError_t run_exact_knn_tc(const XDesc& x, const int32_t* queries, int nq, int k, int32_t* ids, float* dists,
+                             int* err, Arena& ar, cudaStream_t st);
 
 // One set of a batched build, as seen by the output scatter.
 struct BatchSet {
