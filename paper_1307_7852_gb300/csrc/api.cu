@@ -272,9 +272,8 @@ int leaf_stage(knng_handle* h, const TreePlan& P, const DevPlan& dp, const XDesc
     cudaError_t e;
     const int kp = std::min(mult * k, 128);
     if (prec == KNNG_PREC_FP32) {
-        if (!ar.base) return KNNG_OK;
-        e = all_exact ? cudaMemsetAsync(all_exact, 0, sizeof(int), st) : cudaSuccess;
-        if (e == cudaSuccess) e = run_leaf_knn_f32(x, P, dp, T, perm, k, kp, ids, dists, st);
+        e = (all_exact && ar.base) ? cudaMemsetAsync(all_exact, 0, sizeof(int), st) : cudaSuccess;
+        if (e == cudaSuccess) e = run_leaf_knn_f32(x, P, dp, T, perm, k, kp, ids, dists, ar, st);
     } else if (prec == KNNG_PREC_BF16 || prec == KNNG_PREC_FP8E4M3) {
         const auto it = h->tune.find(tc_key(P, x.d, prec));
         const TcTile* tile = it == h->tune.end() ? nullptr : &it->second;

@@ -153,7 +153,7 @@ cudaError_t run_partition(const XDesc& x, const TreePlan& plan, const DevPlan& d
                           int* err = nullptr);
 
 cudaError_t run_leaf_knn_f32(const XDesc& x, const TreePlan& P, const DevPlan& dp, int T,
-                             const int32_t* perm, int k, int kp, int32_t* ids, float* dists,
+                             const int32_t* perm, int k, int kp, int32_t* ids, float* dists, Arena& ar,
                              cudaStream_t st);
 
 // Tile choices of the tensor-core leaf kernel for one problem shape:

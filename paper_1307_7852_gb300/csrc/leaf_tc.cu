@@ -126,7 +126,7 @@ cudaError_t run_leaf_knn_tc(const XDesc& x, const TreePlan& P, const DevPlan& dp
     // (their candidates in [rows][kp] local indices, a flag per leaf)
     const bool staged = leaf_rescore_staged_ok(kp, P.max_leaf);
     const int nleaves = (int)P.leaf_off.size() - 1;
-    uint16_t* cand = staged ? ar.take<uint16_t>((size_t)T * x.n * kp) : nullptr;
+    uint16_t* cand = staged ? ar.take<uint16_t>((size_t)T * x.n * kp + 8) : nullptr;
     uint8_t* leaf_flag = staged ? ar.take<uint8_t>((size_t)T * nleaves) : nullptr;
     if (!ar.base) return cudaSuccess;
     TcGeom G = tc_geometry(P, x.d, prec, tile);
