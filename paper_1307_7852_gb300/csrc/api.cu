@@ -656,7 +656,8 @@ int knng_leaf_knn(knng_handle* h, const void* X, int32_t dtype, int64_t n, int32
     if ((r = ensure_plan(h, n, g, st))) return r;
     Arena m;
     if ((r = leaf_stage(h, h->plan, h->dplan, x, T, perm, k, precision, rescore_mult, ids, dists, m, st))) return r;
-    if ((r = ensure_ws(h, m.off, st))) return r;
+    // (a stage that needs no scratch still runs with a base, not as a measurement)
+    if ((r = ensure_ws(h, std::max<size_t>(m.off, 1), st))) return r;
     Arena a;
     a.base = h->ws;
     return leaf_stage(h, h->plan, h->dplan, x, T, perm, k, precision, rescore_mult, ids, dists, a, st);

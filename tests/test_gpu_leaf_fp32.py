@@ -46,3 +46,13 @@ def test_unaligned_rows_exact():
     buf = torch.zeros(1500 * 53 + 1, device="cuda")
     buf[1:] = dev(X).reshape(-1)
     _check(X, buf[1:].view(1500, 53), 2, 128, 12)
+
+
+@pytest.mark.parametrize("k,mult", [(20, 2), (30, 2)])
+def test_leaf_stage_is_the_first_call_of_a_handle(k, mult):
+    X = np.random.default_rng(6).integers(0, 255, size=(1500, 50)).astype(np.float32)
+    Xd = dev(X)
+    perm = knng().knng_partition(Xd, 1, 128, 3)
+    ids, dd = knng().knng_leaf_knn(Xd, 1, 128, perm, k, 0, mult, h=knng().Handle(0))
+    oi, od = oracle.leaf_knn(X, host(perm)[0], knng().knng_leaf_offsets(1500, 128), k)
+    assert_lists_exact(host(ids)[0], host(dd)[0], oi, od)
