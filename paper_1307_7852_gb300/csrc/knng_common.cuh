@@ -156,6 +156,19 @@ struct RowLoader {
         if (kDT == kDtU8) return bytes_to_float4(load_u8x4(i, j));
         return __ldg(reinterpret_cast<const float4*>(static_cast<const float*>(X) + row_off(i) + j));
     }
+    // four entries at element offset o (of vector-aligned rows)
+    __device__ __forceinline__ float4 load4_at(uint64_t o) const
+    {
+        if (kDT == kDtF16) {
+            const uint2 u = __ldg(reinterpret_cast<const uint2*>(static_cast<const __half*>(X) + o));
+            const float2 fa = __half22float2(*reinterpret_cast<const __half2*>(&u.x));
+            const float2 fb = __half22float2(*reinterpret_cast<const __half2*>(&u.y));
+            return make_float4(fa.x, fa.y, fb.x, fb.y);
+        }
+        if (kDT == kDtU8)
+            return bytes_to_float4(__ldg(reinterpret_cast<const unsigned int*>(static_cast<const uint8_t*>(X) + o)));
+        return __ldg(reinterpret_cast<const float4*>(static_cast<const float*>(X) + o));
+    }
     // bytes j..j+3 of row i packed little-endian (U8 rows, vector-aligned)
     __device__ __forceinline__ uint32_t load_u8x4(int64_t i, int j) const
     {
@@ -163,6 +176,16 @@ struct RowLoader {
     }
     // every load of a row is a full vector load (aligned rows, d % 4 == 0)
     __device__ __forceinline__ bool all_vec() const { return vec && (d & 3) == 0; }
+    // rows scored eight lanes a row (warp_canon_dist_g8): FP32 up to 208
+    // entries, FP16 up to 512.  Both forms read at the L2's rate on wide rows
+    // (about 10 TB/s), where the other one's 512 contiguous bytes a load are
+    // better; one propagation round of 200k points, k = 20, other form -> this
+    // one, ms: FP32 d = 64 2.77 -> 1.73, 128 3.10 -> 2.87, 192 4.42 -> 4.08,
+    // 224 4.57 -> 4.67, 256 4.63 -> 5.31; FP16 128 3.15 -> 2.31, 512 8.89 -> 7.69
+    __host__ __device__ __forceinline__ bool narrow() const
+    {
+        return kDT == kDtF16 ? d <= 512 : kDT == kDtF32 ? d <= 208 : false;
+    }
     // byte rows whose squared distances stay below 2^24 (d * 255^2 < 2^24):
     // every partial sum of the canonical FP32 distance is then an exact
     // integer, so integer arithmetic in any order gives the same value
@@ -670,9 +693,67 @@ __device__ __forceinline__ float warp_canon_dist_batch(const RowLoader<kDT>& L, 
     return out;
 }
 
-// Byte rows with exact integer distances (RowLoader::int_exact): the same
-// lane split and reduction tree as warp_canon_dist_batch in 32-bit integer
-// arithmetic, |x - y| per byte and a 4-way dot product per word.  Equal to
+// Canonical distances from point a to b[0..nb) (nb <= 32, b in shared
+// memory): lane l < nb returns the distance to b[l].  Rows must be
+// vector-aligned with d % 4 == 0.
+// Eight lanes per row and block of 32 entries: lane q of group g loads entries
+// 4q .. 4q + 3 (partial q of the block) of the group's rows b[8g .. 8g + 7],
+// so one load instruction fetches four whole 128-byte blocks, and a row ends
+// with its last block (no padding to 128 entries).  Recursive halving over the
+// group's eight lanes (offsets 4, 2, 1: each lane keeps half of its rows'
+// values and receives its partner's copy of them) performs the additions of
+// the block butterfly and leaves lane q with the block value of row b[8g + q],
+// which it adds to that row's running sum.  Bit-identical to warp_canon_dist:
+// 7 shuffles and 8 loads per block of 32 rows, a rolled loop of one block
+// (two blocks in flight spill: 23.4 -> 28.8 ms on 2M x 96 FP16 rows, where
+// warp_canon_dist_batch, whose 96-entry row pays for 128 and whose two
+// unrolled batches stall on instruction fetch, takes 38.7).
+template <int kDT>
+__device__ __forceinline__ float warp_canon_dist_g8(const RowLoader<kDT>& L, int64_t a, const int* b, int nb)
+{
+    const int lane = threadIdx.x & 31;
+    const int q4 = 4 * (lane & 7), g8 = lane & ~7;
+    uint64_t off[8];
+#pragma unroll
+    for (int r = 0; r < 8; ++r) off[r] = L.row_off(g8 + r < nb ? b[g8 + r] : (int)a) + q4;
+    const uint64_t offa = L.row_off(a) + q4;
+    float tot = 0.f;
+#pragma unroll 1
+    for (int j0 = 0; j0 < L.d; j0 += 32) {
+        float p[8];
+#pragma unroll
+        for (int r = 0; r < 8; ++r) p[r] = 0.f;
+        if (j0 + q4 < L.d) {
+            const float4 xa = L.load4_at(offa + j0);
+            float4 u[8];
+#pragma unroll
+            for (int r = 0; r < 8; ++r) u[r] = L.load4_at(off[r] + j0);
+            const float2 na = make_float2(-xa.x, -xa.y), nb2 = make_float2(-xa.z, -xa.w);
+#pragma unroll
+            for (int r = 0; r < 8; ++r) {
+                // (packed subtractions: each half rounds like the scalar one)
+                const float2 lo = __fadd2_rn(make_float2(u[r].x, u[r].y), na);
+                const float2 hi = __fadd2_rn(make_float2(u[r].z, u[r].w), nb2);
+                p[r] = fmaf(hi.y, hi.y, fmaf(hi.x, hi.x, fmaf(lo.y, lo.y, lo.x * lo.x)));
+            }
+        }
+#pragma unroll
+        for (int o = 4; o >= 1; o >>= 1) {
+            const bool hi = (lane & o) != 0;
+#pragma unroll
+            for (int i = 0; i < o; ++i) {
+                const float send = hi ? p[i] : p[i + o];
+                const float keep = hi ? p[i + o] : p[i];
+                p[i] = keep + __shfl_xor_sync(KNNG_FULL_MASK, send, o);
+            }
+        }
+        tot = tot + p[0];
+    }
+    return tot;
+}
+
+// Byte rows with exact integer distances (RowLoader::int_exact): a lane takes
+// entries 128c + 4l .. +3 of W rows in 32-bit integer arithmetic, |x - y| per byte and a 4-way dot product per word.  Equal to
 // the canonical FP32 distance, since every partial sum of that one is exact.
 template <int W, int kDT>
 __device__ __forceinline__ float warp_u8_dist_batch(const RowLoader<kDT>& L, int64_t a, const int* b, int nb)
@@ -775,11 +856,25 @@ __device__ __forceinline__ void score_u8_g8(const uint8_t* X, int64_t ld, int d,
 
 // Canonical distances from a to b[0..nb) (nb <= 32): lane c < nb returns the
 // distance to b[c].  Byte rows with exact integer distances take one batch
-// of 32 (32 rows in flight per warp), other rows two batches of 16.
-template <int kDT>
+// of 32 (32 rows in flight per warp), other vector-aligned rows eight lanes a
+// row, the rest one distance at a time.
+// kForm: 0 picks by the row width here, 1 / 2 are kernels built for narrow /
+// other rows (the code of one form only: with both, the propagation of
+// 256-entry rows ran 3 % slower).
+template <int kForm = 0, int kDT = 0>
 __device__ __forceinline__ float warp_canon_dist32(const RowLoader<kDT>& L, int64_t a, const int* b, int nb)
 {
     if (kDT == kDtU8 && L.all_vec() && L.int_exact()) return warp_u8_dist_batch<32>(L, a, b, nb);
+    if (kForm != 2 && L.all_vec() && (kForm == 1 || L.narrow())) return warp_canon_dist_g8(L, a, b, nb);
+    if (kForm == 1) {
+        const int lane = threadIdx.x & 31;
+        float mine = 0.f;
+        for (int c = 0; c < nb; ++c) {
+            const float dd = warp_canon_dist(L, a, b[c]);
+            if (lane == c) mine = dd;
+        }
+        return mine;
+    }
     const int lane = threadIdx.x & 31;
     const float lo = warp_canon_dist16(L, a, b, min(nb, 16));
     float hi = 0.f;

@@ -45,7 +45,8 @@ BfLayout bf_layout(int budget)
 }
 }  // namespace
 
-template <int kDT>
+// kForm: the scoring of rows that are not bytes, see warp_canon_dist32.
+template <int kDT, int kForm>
 __global__ void __launch_bounds__(256, 2) propagate_bf_kernel(RowLoader<kDT> L, RowLoader<kDtU8> Lb,
                                                               const int* __restrict__ xb_bad, int64_t n, int k,
                                                               int budget, const int32_t* __restrict__ order,
@@ -90,7 +91,7 @@ __global__ void __launch_bounds__(256, 2) propagate_bf_kernel(RowLoader<kDT> L, 
                 const int nb = min(32, end - c0);
                 float dd;
                 if (kDT == kDtF32 && bytes) dd = warp_canon_dist32(Lb, p, vid + c0, nb);
-                else dd = warp_canon_dist32(L, p, vid + c0, nb);
+                else dd = warp_canon_dist32<kForm>(L, p, vid + c0, nb);
                 if (lane < nb) vkey[c0 + lane] = pack_key(dd, (uint32_t)vid[c0 + lane]);
             }
             cnt = end;
@@ -156,7 +157,9 @@ cudaError_t run_propagate_best_first(const XDesc& x, int k, int budget, const in
     cudaError_t e = cudaSuccess;
     auto launch = [&](auto dt) {
         constexpr int kDT = decltype(dt)::value;
-        auto kern = propagate_bf_kernel<kDT>;
+        RowLoader<kDT> rl{x.X, x.ld, x.d, x.vec};
+        auto kern = propagate_bf_kernel<kDT, 2>;
+        if (rl.narrow()) kern = propagate_bf_kernel<kDT, kDT == kDtU8 ? 2 : 1>;
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return;
         int per_sm = 0;
@@ -165,7 +168,6 @@ cudaError_t run_propagate_best_first(const XDesc& x, int k, int budget, const in
         int64_t blocks = (int64_t)num_sms() * per_sm;
         const int64_t need = (x.n + warps - 1) / warps;
         if (blocks > need) blocks = need;
-        RowLoader<kDT> rl{x.X, x.ld, x.d, x.vec};
         const RowLoader<kDtU8> rb{x.Xb, x.ldb, x.d, true};
         kern<<<(int)blocks, warps * 32, smem, st>>>(rl, rb, x.xb_bad, x.n, k, budget, order, ids_in, ids, dists,
                                                     BL.H, BL.hshift, BL.Bc, (int)BL.per_warp);
