@@ -33,12 +33,14 @@ struct Chunk {
     int32_t first;  // index of the node's first chunk in the level's chunk list
 };
 
+// State of a large node's radix select: the digits found so far (in the end
+// the median key), the rank among the keys with that prefix (in the end how
+// many of the keys equal to the median go left), the blocks' ticket.
 struct SelState {
-    unsigned long long prefix;
-    unsigned long long mask;
-    unsigned long long thr;
+    uint32_t prefix;
     int32_t rank;
-    int32_t done;
+    uint32_t ticket;
+    uint32_t pad;
 };
 
 constexpr int kSmallCap = 8192;    // nodes up to this size split in one block

@@ -9,10 +9,11 @@
 //                    projects it on the direction of its node in every tree
 //                    (fixed-order FP32, bit-identical to the CPU definition);
 //                    the 32-bit key lands at the point's current position.
-//   3. select     -- per node, the floor(m/2)-th smallest 64-bit key
-//                    (ord(s) << 32 | id) by radix select: one block per node
-//                    for nodes <= kSmallCap, otherwise block-private
-//                    histograms merged in global memory, one digit per pass.
+//   3. select     -- per node, the floor(m/2)-th smallest (key, id) by radix
+//                    select on the keys (equal keys in position order, which
+//                    is id order): one block per node for nodes <= kSmallCap,
+//                    otherwise block-private histograms merged in global
+//                    memory, three digits.
 //   4. scatter    -- stable partition of each node into its two children.
 // Stability makes every node's segment ascend by id, so the leaves come out
 // in canonical order without a final sort.
@@ -167,20 +168,33 @@ __global__ void init_root_nodes_kernel(int64_t n, const SplitNode* __restrict__ 
     }
 }
 
-// dirs[t][s][0..d_pad): direction of split node s of this level in tree
-// t0 + t (a tree's directions depend on its own index only).
-__global__ void gen_dirs_kernel(float* dirs, int T, int S, int d, int d_pad,
-                                const SplitNode* nodes, uint32_t level, uint64_t seed, uint32_t t0)
+// Directions of a run of levels in one launch (one per level costs a small
+// build 3 us each): level by level, dirs[t][s][0..d_pad) of split node s in
+// tree t0 + t (a tree's directions depend on its own index only).
+constexpr int kMaxDirLevels = 32;
+struct DirLevels {
+    int count;
+    uint32_t first;                  // number of the run's first level
+    int S[kMaxDirLevels];            // split nodes
+    int64_t node_base[kMaxDirLevels];
+    int64_t end[kMaxDirLevels];      // first direction (t, s) past the level, over the run
+};
+__global__ void gen_dirs_kernel(float* dirs, int d, int d_pad, const SplitNode* __restrict__ nodes,
+                                const __grid_constant__ DirLevels lv, uint64_t seed, uint32_t t0)
 {
     const int q4 = d_pad / 4;
-    const int64_t total = (int64_t)T * S * q4;
+    const int64_t total = lv.end[lv.count - 1] * q4;
     const uint2 key = make_uint2((uint32_t)(seed & 0xFFFFFFFFu), (uint32_t)(seed >> 32));
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
          e += (int64_t)gridDim.x * blockDim.x) {
-        const int q = (int)(e % q4);
-        const int s = (int)((e / q4) % S);
-        const int t = (int)(e / ((int64_t)q4 * S));
-        const uint4 w = philox4x32_10(make_uint4(t0 + (uint32_t)t, level, nodes[s].v, (uint32_t)q), key);
+        const int64_t dir = e / q4;
+        const int q = (int)(e - dir * q4);
+        int l = 0;
+        while (dir >= lv.end[l]) ++l;
+        const int64_t in = dir - (l ? lv.end[l - 1] : 0);
+        const int t = (int)(in / lv.S[l]), s = (int)(in - (int64_t)t * lv.S[l]);
+        const uint4 w = philox4x32_10(
+            make_uint4(t0 + (uint32_t)t, lv.first + (uint32_t)l, nodes[lv.node_base[l] + s].v, (uint32_t)q), key);
         const int j = 4 * q;
         float4 a;
         a.x = (j + 0 < d) ? tri_entry(w.x) : 0.f;
@@ -192,16 +206,19 @@ __global__ void gen_dirs_kernel(float* dirs, int T, int S, int d, int d_pad,
 }
 
 // Learned splits, step 1: range (as order keys) of every tree's feature of
-// this level inside every node.  Positions are visited in node order, so the
-// lanes of a warp nearly always share one node: the warp then reduces its
-// keys and one lane updates the node's range (on the top levels every point
-// of a tree would otherwise hit the same two words).
+// this level inside every node, and the feature's keys themselves (the
+// projection replaces those of the nodes whose feature is flat).  Positions
+// are visited in node order, so the lanes of a warp nearly always share one
+// node: the warp then reduces its keys and one lane updates the node's range
+// (on the top levels every point of a tree would otherwise hit the same two
+// words).
 struct FeatOfTree {
     int f[32];
 };
 __global__ void node_feature_range_kernel(int64_t n, int T, const float* __restrict__ Z, int C, FeatOfTree ft,
                                           const int32_t* __restrict__ node_pos, const int32_t* __restrict__ perm,
-                                          int S, uint32_t* __restrict__ rmin, uint32_t* __restrict__ rmax)
+                                          int S, uint32_t* __restrict__ rmin, uint32_t* __restrict__ rmax,
+                                          uint32_t* __restrict__ keys)
 {
     const int64_t total = (int64_t)T * n;
     const int lane = threadIdx.x & 31;
@@ -216,6 +233,7 @@ __global__ void node_feature_range_kernel(int64_t n, int T, const float* __restr
                 const int t = (int)(e / n);
                 key = (int64_t)t * S + sn;
                 o = ord_key(Z[(int64_t)perm[e] * C + ft.f[t]]);
+                keys[e] = o;
             }
         }
         const int64_t key0 = __shfl_sync(KNNG_FULL_MASK, key, 0);
@@ -279,14 +297,27 @@ cudaError_t run_feature_range(const float* Z, int64_t n, int C, uint32_t* mm, fl
 
 // Learned-split settings of one level, passed to the projection kernel.
 struct LevelFeat {
-    const float* Z;
-    int C;
     FeatOfTree ft;
     const uint32_t* rmin;
     const uint32_t* rmax;
     const float* frange;
     float tau;
+    const int* any_flat;  // nonzero: some node of the level needs the projection
+    // a node splits on its learned feature while the feature still varies there
+    __device__ __forceinline__ bool varies(int t, int64_t node) const
+    {
+        const float span = unord_key(rmax[node]) - unord_key(rmin[node]);
+        return span > tau * frange[ft.f[t]];
+    }
 };
+
+// Step 2: whether any node of the level has a flat feature (*any must be 0).
+__global__ void learned_flat_kernel(int T, int S, LevelFeat lv, int* any)
+{
+    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const bool flat = e < (int64_t)T * S && !lv.varies((int)(e / S), e);
+    if (__syncthreads_or(flat) && threadIdx.x == 0) *any = 1;
+}
 
 void learned_feature_order(uint64_t seed, int T, int C, LearnedFeat& lf)
 {
@@ -323,26 +354,14 @@ __device__ __forceinline__ void project_body(const Loader& L, int64_t n, int T, 
             const int tl = t0 + lane;
             const int my_s = (lane < 8 && tl < T) ? node_of[(int64_t)tl * n + i] : -1;
             if (__ballot_sync(KNNG_FULL_MASK, my_s >= 0) == 0) continue;
-            // learned levels: a node splits on its learned feature while the
-            // feature still varies there, and then needs no projection
-            bool my_feat = false;
-            if (kLearned && my_s >= 0) {
-                const int f = lv.ft.f[tl];
-                const int64_t ns = (int64_t)tl * S + my_s;
-                const float span = unord_key(lv.rmax[ns]) - unord_key(lv.rmin[ns]);
-                my_feat = span > lv.tau * lv.frange[f];
-            }
-            const int proj_s = my_feat ? -1 : my_s;
+            // learned levels: a node that splits on its learned feature has
+            // its keys and needs no projection
+            int proj_s = my_s;
+            if (kLearned && my_s >= 0 && lv.varies(tl, (int64_t)tl * S + my_s)) proj_s = -1;
+            if (kLearned && __ballot_sync(KNNG_FULL_MASK, proj_s >= 0) == 0) continue;
             int sv[8];
 #pragma unroll
             for (int u = 0; u < 8; ++u) sv[u] = __shfl_sync(KNNG_FULL_MASK, proj_s, u);
-            if (kLearned && __ballot_sync(KNNG_FULL_MASK, proj_s >= 0) == 0) {
-                if (my_s >= 0) {
-                    const int64_t row = (int64_t)tl * n;
-                    keys[row + pos_of[row + i]] = ord_key(lv.Z[i * lv.C + lv.ft.f[tl]]);
-                }
-                continue;
-            }
             float acc[8];
 #pragma unroll
             for (int u = 0; u < 8; ++u) acc[u] = 0.0f;
@@ -373,10 +392,9 @@ __device__ __forceinline__ void project_body(const Loader& L, int64_t n, int T, 
                 for (int o = 16; o >= 1; o >>= 1) acc[u] += __shfl_xor_sync(KNNG_FULL_MASK, acc[u], o);
                 if (lane == u) mine = acc[u];
             }
-            if (my_s >= 0) {
+            if (proj_s >= 0) {
                 const int64_t row = (int64_t)tl * n;
-                const uint32_t key = my_feat ? ord_key(lv.Z[i * lv.C + lv.ft.f[tl]]) : ord_key(mine);
-                keys[row + pos_of[row + i]] = key;
+                keys[row + pos_of[row + i]] = ord_key(mine);
             }
         }
     }
@@ -393,6 +411,7 @@ __global__ void __launch_bounds__(256) project_kernel(RowLoader<kDT> L, RowLoade
                                                       const int32_t* __restrict__ pos_of,
                                                       uint32_t* __restrict__ keys, LevelFeat lv)
 {
+    if (kLearned && *lv.any_flat == 0) return;
     if constexpr (kDT == kDtF32) {
         if (xb_bad && *xb_bad == 0) {
             if (bytes_elsewhere) return;
@@ -661,59 +680,10 @@ __global__ void __launch_bounds__(256, 4) project_bytes_tma_kernel(const __grid_
     }
 }
 
-// ---- block radix select (one block, keys in shared memory) ---------------
-template <int NT>
-__device__ unsigned long long block_select(const unsigned long long* k64, int m, int want,
-                                           uint32_t* hist, uint32_t* bcast)
-{
-    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    unsigned long long prefix = 0, mask = 0;
-    int rank = want;
-    for (int shift = 56;; shift -= 8) {
-        for (int b = tid; b < 256; b += NT) hist[b] = 0;
-        __syncthreads();
-        for (int e = tid; e < m; e += NT) {
-            const unsigned long long kv = k64[e];
-            if ((kv & mask) == prefix) atomicAdd(&hist[(kv >> shift) & 0xFF], 1u);
-        }
-        __syncthreads();
-        if (w == 0) {
-            uint32_t c[8], lsum = 0;
-#pragma unroll
-            for (int b = 0; b < 8; ++b) { c[b] = hist[lane * 8 + b]; lsum += c[b]; }
-            uint32_t incl = lsum;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t t = __shfl_up_sync(KNNG_FULL_MASK, incl, o);
-                if (lane >= o) incl += t;
-            }
-            const uint32_t excl = incl - lsum;
-            if (excl < (uint32_t)rank && (uint32_t)rank <= incl) {
-                uint32_t run = excl;
-                bool found = false;
-#pragma unroll
-                for (int b = 0; b < 8; ++b) {
-                    if (!found && run < (uint32_t)rank && (uint32_t)rank <= run + c[b]) {
-                        bcast[0] = lane * 8 + b;
-                        bcast[1] = run;
-                        bcast[2] = c[b];
-                        found = true;
-                    }
-                    run += c[b];
-                }
-            }
-        }
-        __syncthreads();
-        const uint32_t digit = bcast[0], before = bcast[1], inbin = bcast[2];
-        prefix |= (unsigned long long)digit << shift;
-        mask |= 0xFFull << shift;
-        rank -= (int)before;
-        __syncthreads();
-        if ((uint32_t)rank == inbin || shift == 0)
-            return prefix | (shift ? ((1ull << shift) - 1) : 0ull);
-    }
-}
-
+// The median split works on the 32-bit keys alone.  The order (key, id) is the
+// order (key, position) -- a node's positions ascend by id -- so the left child
+// is: the keys below the floor(m/2)-th smallest, and of the keys equal to it
+// the first `take` in position order.
 // Exclusive block scan of one int per thread; returns the prefix, and the
 // total in *total.
 template <int NT>
@@ -746,52 +716,104 @@ __device__ int block_excl_scan(int v, int* sh, int* total)
     return r;
 }
 
-// Stable two-way scatter of elements [0, len) of a slice (keys in shared
-// memory) in rounds of NT consecutive elements: a block-wide count of the
-// left elements before each one gives its destination, so a warp's left and
-// right elements land in two contiguous runs.  lbase/rbase: destination of
-// the slice's first left / right element.  The node of every destination
-// position is written to node_pos; the maps by id (pos_of, node_of) only
-// when a later projection reads them (id_maps).
-template <int NT>
-__device__ void stable_scatter(const unsigned long long* k64, int len, unsigned long long thr,
-                               int32_t lbase, int32_t rbase, int32_t childL, int32_t childR,
-                               int32_t* perm_nxt, int32_t* node_pos, int32_t* pos_of, int32_t* node_of,
-                               bool id_maps, int* sh)
+// ---- block radix select (one block, keys in shared memory) ---------------
+// The want-th smallest of k32[0..m) (1 <= want <= m) and, in *take, how many of
+// the keys equal to it belong to the want smallest.  The bits that all keys
+// share are skipped; the rest is resolved B bits a pass.  hist: 2^B words.
+template <int NT, int B>
+__device__ uint32_t block_select(const uint32_t* k32, int m, int want, uint32_t* hist, int* sh, int* take)
 {
-    constexpr int NW = NT / 32;
-    static_assert(NW <= 16, "two rounds of warp counts share sh[0..31]");
+    constexpr int PER = (1 << B) / NT;  // bins per thread
+    __shared__ uint32_t ends[2][NT / 32];
+    __shared__ int pick[2];
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    int before = 0;  // left elements of the earlier rounds
-    for (int base = 0, r = 0; base < len; base += NT, r ^= 1) {
-        const int e = base + tid;
-        const unsigned long long kv = e < len ? k64[e] : ~0ull;
-        const bool left = e < len && kv <= thr;
-        const uint32_t b = __ballot_sync(KNNG_FULL_MASK, left);
-        // the counts alternate between two halves of sh: one barrier a round
-        if (lane == 0) sh[16 * r + w] = __popc(b);
-        __syncthreads();
-        int pre = 0, tot = 0;
+    uint32_t mn = 0xFFFFFFFFu, mx = 0u;
+    for (int e = tid; e < m; e += NT) {
+        mn = min(mn, k32[e]);
+        mx = max(mx, k32[e]);
+    }
+    mn = __reduce_min_sync(KNNG_FULL_MASK, mn);
+    mx = __reduce_max_sync(KNNG_FULL_MASK, mx);
+    if (lane == 0) {
+        ends[0][w] = mn;
+        ends[1][w] = mx;
+    }
+    __syncthreads();
 #pragma unroll
-        for (int i = 0; i < NW; ++i) {
-            const int c = sh[16 * r + i];
-            pre += i < w ? c : 0;
-            tot += c;
+    for (int i = 0; i < NT / 32; ++i) {
+        mn = min(mn, ends[0][i]);
+        mx = max(mx, ends[1][i]);
+    }
+    int hi = mn == mx ? 0 : 32 - __clz((int)(mn ^ mx));  // bits [hi, 32) are common
+    uint32_t prefix = hi >= 32 ? 0u : (mn >> hi) << hi;
+    int rank = want;
+    while (hi > 0) {
+        const int lo = max(0, hi - B);
+        const uint32_t dmask = (1u << (hi - lo)) - 1u;
+        for (int b = tid; b < (1 << B); b += NT) hist[b] = 0;
+        __syncthreads();
+        for (int e = tid; e < m; e += NT) {
+            const uint32_t kv = k32[e];
+            if (hi >= 32 || ((kv ^ prefix) >> hi) == 0u) atomicAdd(&hist[(kv >> lo) & dmask], 1u);
         }
-        if (e < len) {
-            const int lrank = before + pre + __popc(b & lanemask_lt());
-            const int32_t id = (int32_t)(uint32_t)kv;
-            const int32_t dst = left ? lbase + lrank : rbase + (e - lrank);
-            const int32_t child = left ? childL : childR;
-            perm_nxt[dst] = id;
-            node_pos[dst] = child;
-            if (id_maps) {
-                pos_of[id] = dst;
-                node_of[id] = child;
+        __syncthreads();
+        uint32_t cb[PER];
+        int sum = 0;
+#pragma unroll
+        for (int b = 0; b < PER; ++b) {
+            cb[b] = hist[tid * PER + b];
+            sum += (int)cb[b];
+        }
+        int total;
+        int run = block_excl_scan<NT>(sum, sh, &total);
+        if (run < rank && rank <= run + sum) {
+#pragma unroll
+            for (int b = 0; b < PER; ++b) {
+                if (run < rank && rank <= run + (int)cb[b]) {
+                    pick[0] = tid * PER + b;
+                    pick[1] = rank - run;
+                }
+                run += (int)cb[b];
             }
         }
-        before += tot;
+        __syncthreads();
+        prefix |= (uint32_t)pick[0] << lo;
+        rank = pick[1];
+        hi = lo;
     }
+    *take = rank;
+    return prefix;
+}
+
+// Stable two-way scatter, one round of NT consecutive elements: `less` / `equal`
+// mark the elements below / equal to the median key.  Returns the number of
+// left elements before this one, given the counts of smaller and equal
+// elements before the round (advanced over it), and whether it is left.
+// sh: 2 x NT / 32 words, halves used in turn (r = round).
+template <int NT>
+__device__ __forceinline__ int split_round(bool less, bool equal, int take, int r, int* sh, int& less_before,
+                                           int& equal_before, bool& left)
+{
+    constexpr int NW = NT / 32;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const uint32_t bl = __ballot_sync(KNNG_FULL_MASK, less), be = __ballot_sync(KNNG_FULL_MASK, equal);
+    // the counts alternate between two halves of sh: one barrier a round
+    if (lane == 0) sh[NW * (r & 1) + w] = __popc(bl) | (__popc(be) << 16);
+    __syncthreads();
+    int pre = 0, tot = 0;
+#pragma unroll
+    for (int i = 0; i < NW; ++i) {
+        const int v = sh[NW * (r & 1) + i];
+        pre += i < w ? v : 0;
+        tot += v;
+    }
+    const uint32_t lt = lanemask_lt();
+    const int lb = less_before + (pre & 0xFFFF) + __popc(bl & lt);
+    const int eb = equal_before + (pre >> 16) + __popc(be & lt);
+    left = less || (equal && eb < take);
+    less_before += tot & 0xFFFF;
+    equal_before += tot >> 16;
+    return lb + min(eb, take);
 }
 
 // Whether this level's scatter keeps the maps by id: 1 always, 0 never,
@@ -802,164 +824,163 @@ __device__ __forceinline__ bool want_id_maps(int id_mode, const int* xb_bad)
     return id_mode == 1 || (id_mode == 2 && xb_bad && *xb_bad != 0);
 }
 
-// One block per (split node, tree), node <= kSmallCap points.
-template <int NT>
+// One block per (split node, tree), node <= kSmallCap points.  What bounds it:
+// the chain of barriers (select passes, scatter rounds), so small nodes take
+// small blocks -- more of them resident -- and few bins.
+template <int NT, int B>
 __global__ void __launch_bounds__(NT) split_small_kernel(int64_t n, const SplitNode* __restrict__ nodes,
                                                          const uint32_t* __restrict__ keys,
                                                          const int32_t* __restrict__ perm_cur,
                                                          int32_t* perm_nxt, int32_t* node_pos, int32_t* pos_of,
                                                          int32_t* node_of, int id_mode, const int* xb_bad)
 {
-    extern __shared__ unsigned long long k64[];
-    __shared__ uint32_t hist[256];
-    __shared__ uint32_t bcast[4];
+    extern __shared__ uint32_t k32[];
+    __shared__ uint32_t hist[1 << B];
     __shared__ int sh[33];
     const SplitNode nd = nodes[blockIdx.x];
     const int64_t row = (int64_t)blockIdx.y * n;
     const int m = nd.size;
-    for (int e = threadIdx.x; e < m; e += NT)
-        k64[e] = ((unsigned long long)keys[row + nd.off + e] << 32) | (uint32_t)perm_cur[row + nd.off + e];
+    for (int e = threadIdx.x; e < m; e += NT) k32[e] = keys[row + nd.off + e];
     __syncthreads();
-    const unsigned long long thr = block_select<NT>(k64, m, m / 2, hist, bcast);
-    stable_scatter<NT>(k64, m, thr, nd.off, nd.off + m / 2, nd.childL, nd.childR, perm_nxt + row,
-                       node_pos + row, pos_of + row, node_of + row, want_id_maps(id_mode, xb_bad), sh);
+    int take;
+    const uint32_t thr = block_select<NT, B>(k32, m, m / 2, hist, sh, &take);
+    __syncthreads();
+    const bool id_maps = want_id_maps(id_mode, xb_bad);
+    int lb = 0, eb = 0;
+    for (int base = 0, r = 0; base < m; base += NT, ++r) {
+        const int e = base + threadIdx.x;
+        const bool live = e < m;
+        const int32_t id = live ? perm_cur[row + nd.off + e] : 0;
+        const uint32_t kv = live ? k32[e] : 0xFFFFFFFFu;
+        bool left;
+        const int before = split_round<NT>(live && kv < thr, live && kv == thr, take, r, sh, lb, eb, left);
+        if (live) {
+            const int32_t dst = left ? nd.off + before : nd.off + m / 2 + (e - before);
+            const int32_t child = left ? nd.childL : nd.childR;
+            perm_nxt[row + dst] = id;
+            node_pos[row + dst] = child;
+            if (id_maps) {
+                pos_of[row + id] = dst;
+                node_of[row + id] = child;
+            }
+        }
+    }
 }
 
 // ---- multi-block split of large nodes ------------------------------------
-__global__ void big_init_kernel(int S, int T, const SplitNode* nodes, SelState* st)
+// Three histogram passes over 11, 11 and 10 bits of the key; the last block of
+// a node to finish a pass picks its digit (no separate launch), then counts
+// per slice and one scatter.  (Eight passes over the 64-bit (key, id) with a
+// pick launch each took 165 us a level at 8 x 1M points, 21 launches; now
+// 118 us, 5 launches.)
+constexpr int kBigBins = 2048;
+
+// Whether this block is the last of the node's `blocks` to get here (every
+// thread's earlier writes are visible to the last one); resets the ticket.
+__device__ __forceinline__ bool last_block(uint32_t* ticket, int blocks)
 {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= S * T) return;
-    SelState s;
-    s.prefix = 0;
-    s.mask = 0;
-    s.thr = 0;
-    s.rank = nodes[e % S].size / 2;
-    s.done = 0;
-    st[e] = s;
+    __shared__ int is_last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const bool l = atomicAdd(ticket, 1u) == (uint32_t)blocks - 1u;
+        if (l) *ticket = 0u;
+        is_last = l;
+    }
+    __syncthreads();
+    if (is_last) __threadfence();
+    return is_last != 0;
 }
 
 template <int NT>
-__global__ void __launch_bounds__(NT) big_hist_kernel(int64_t n, int shift, int S, const Chunk* __restrict__ chunks,
-                                                      const uint32_t* __restrict__ keys,
-                                                      const int32_t* __restrict__ perm,
-                                                      const SelState* __restrict__ st, uint32_t* ghist)
+__global__ void __launch_bounds__(NT) big_hist_kernel(int64_t n, int lo, int bits, int S,
+                                                      const Chunk* __restrict__ chunks,
+                                                      const SplitNode* __restrict__ nodes,
+                                                      const uint32_t* __restrict__ keys, SelState* st, uint32_t* ghist)
 {
-    __shared__ uint32_t h[256];
-    const Chunk c = chunks[blockIdx.x];
-    const int t = blockIdx.y;
-    const SelState s = st[(int64_t)t * S + c.node];
-    if (s.done) return;
-    for (int b = threadIdx.x; b < 256; b += NT) h[b] = 0;
-    __syncthreads();
-    const int64_t base = (int64_t)t * n + c.start;
-    for (int e = threadIdx.x; e < c.len; e += NT) {
-        const unsigned long long kv = ((unsigned long long)keys[base + e] << 32) | (uint32_t)perm[base + e];
-        if ((kv & s.mask) == s.prefix) atomicAdd(&h[(kv >> shift) & 0xFF], 1u);
-    }
-    __syncthreads();
-    uint32_t* g = ghist + ((int64_t)t * S + c.node) * 256;
-    for (int b = threadIdx.x; b < 256; b += NT)
-        if (h[b]) atomicAdd(&g[b], h[b]);
-}
-
-// One warp per (node, tree): choose the digit of this pass.
-__global__ void big_pick_kernel(int shift, int S, SelState* st, uint32_t* ghist)
-{
-    const int lane = threadIdx.x;
-    const int64_t e = (int64_t)blockIdx.y * S + blockIdx.x;
-    SelState s = st[e];
-    if (s.done) return;
-    uint32_t* h = ghist + e * 256;
-    uint32_t c[8], lsum = 0;
-#pragma unroll
-    for (int b = 0; b < 8; ++b) { c[b] = h[lane * 8 + b]; lsum += c[b]; h[lane * 8 + b] = 0; }
-    uint32_t incl = lsum;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t t = __shfl_up_sync(KNNG_FULL_MASK, incl, o);
-        if (lane >= o) incl += t;
-    }
-    const uint32_t excl = incl - lsum;
-    const uint32_t rank = (uint32_t)s.rank;
-    const bool mine = excl < rank && rank <= incl;
-    const uint32_t owner = __ffs(__ballot_sync(KNNG_FULL_MASK, mine)) - 1;
-    uint32_t digit = 0, before = 0, inbin = 0;
-    if (mine) {
-        uint32_t run = excl;
-        bool found = false;
-#pragma unroll
-        for (int b = 0; b < 8; ++b) {
-            if (!found && run < rank && rank <= run + c[b]) {
-                digit = lane * 8 + b; before = run; inbin = c[b]; found = true;
-            }
-            run += c[b];
-        }
-    }
-    digit = __shfl_sync(KNNG_FULL_MASK, digit, owner);
-    before = __shfl_sync(KNNG_FULL_MASK, before, owner);
-    inbin = __shfl_sync(KNNG_FULL_MASK, inbin, owner);
-    if (lane == 0) {
-        s.prefix |= (unsigned long long)digit << shift;
-        s.mask |= 0xFFull << shift;
-        s.rank -= (int)before;
-        if ((uint32_t)s.rank == inbin || shift == 0) {
-            s.done = 1;
-            s.thr = s.prefix | (shift ? ((1ull << shift) - 1) : 0ull);
-        }
-        st[e] = s;
-    }
-}
-
-template <int NT>
-__global__ void __launch_bounds__(NT) big_count_kernel(int64_t n, int S, int nchunks, const Chunk* __restrict__ chunks,
-                                                       const uint32_t* __restrict__ keys,
-                                                       const int32_t* __restrict__ perm,
-                                                       const SelState* __restrict__ st, int32_t* cnt)
-{
+    constexpr int PER = kBigBins / NT;
+    __shared__ uint32_t h[kBigBins];
     __shared__ int sh[33];
     const Chunk c = chunks[blockIdx.x];
     const int t = blockIdx.y;
-    const unsigned long long thr = st[(int64_t)t * S + c.node].thr;
-    const int64_t base = (int64_t)t * n + c.start;
-    int v = 0;
+    SelState* sp = st + (int64_t)t * S + c.node;
+    const int hi = lo + bits;
+    const uint32_t dmask = (1u << bits) - 1u, prefix = hi >= 32 ? 0u : sp->prefix;
+    for (int b = threadIdx.x; b < kBigBins; b += NT) h[b] = 0;
+    __syncthreads();
+    const uint32_t* kp = keys + (int64_t)t * n + c.start;
     for (int e = threadIdx.x; e < c.len; e += NT) {
-        const unsigned long long kv = ((unsigned long long)keys[base + e] << 32) | (uint32_t)perm[base + e];
-        v += kv <= thr;
+        const uint32_t kv = kp[e];
+        if (hi >= 32 || ((kv ^ prefix) >> hi) == 0u) atomicAdd(&h[(kv >> lo) & dmask], 1u);
+    }
+    __syncthreads();
+    uint32_t* g = ghist + ((int64_t)t * S + c.node) * kBigBins;
+    for (int b = threadIdx.x; b < kBigBins; b += NT)
+        if (h[b]) atomicAdd(&g[b], h[b]);
+    const int size = nodes[c.node].size;
+    if (!last_block(&sp->ticket, (size + kChunk - 1) / kChunk)) return;
+    const int rank = hi >= 32 ? size / 2 : sp->rank;
+    uint32_t cb[PER];
+    int sum = 0;
+#pragma unroll
+    for (int b = 0; b < PER; ++b) {
+        cb[b] = __ldcg(&g[threadIdx.x * PER + b]);
+        sum += (int)cb[b];
+        g[threadIdx.x * PER + b] = 0u;  // for the next pass
     }
     int total;
-    block_excl_scan<NT>(v, sh, &total);
-    if (threadIdx.x == 0) cnt[(int64_t)t * nchunks + blockIdx.x] = total;
+    int run = block_excl_scan<NT>(sum, sh, &total);
+    if (run < rank && rank <= run + sum) {
+#pragma unroll
+        for (int b = 0; b < PER; ++b) {
+            if (run < rank && rank <= run + (int)cb[b]) {
+                sp->prefix = prefix | ((uint32_t)(threadIdx.x * PER + b) << lo);
+                sp->rank = rank - run;
+            }
+            run += (int)cb[b];
+        }
+    }
 }
 
-// One block per (node, tree): exclusive scan of the node's chunk counts
-// (in place: counts in, left-destination offsets out), NT chunks at a time.
-// A node's chunks are contiguous in the level's chunk list; its first and
-// its end are found by bisection.
+// Counts of smaller and equal keys per slice; the node's last block turns them
+// into the counts before each slice (cnt[.][0] and [1]).
 template <int NT>
-__global__ void __launch_bounds__(NT) big_base_kernel(int S, int nchunks, const Chunk* __restrict__ chunks,
-                                                      int32_t* cnt_to_base)
+__global__ void __launch_bounds__(NT) big_count_kernel(int64_t n, int S, int nchunks, const Chunk* __restrict__ chunks,
+                                                       const SplitNode* __restrict__ nodes,
+                                                       const uint32_t* __restrict__ keys, SelState* st, int2* cnt)
 {
     __shared__ int sh[33];
-    const int s = blockIdx.x, t = blockIdx.y;
-    auto first_of = [&](int node) {
-        int lo = 0, hi = nchunks;
-        while (lo < hi) {
-            const int mid = (lo + hi) / 2;
-            if (chunks[mid].node < node) lo = mid + 1; else hi = mid;
+    const Chunk c = chunks[blockIdx.x];
+    const int t = blockIdx.y;
+    SelState* sp = st + (int64_t)t * S + c.node;
+    const uint32_t thr = sp->prefix;
+    const uint32_t* kp = keys + (int64_t)t * n + c.start;
+    int v = 0, q = 0;
+    for (int e = threadIdx.x; e < c.len; e += NT) {
+        const uint32_t kv = kp[e];
+        v += kv < thr;
+        q += kv == thr;
+    }
+    int total;
+    block_excl_scan<NT>(v | (q << 16), sh, &total);  // (a slice has 4,096 points)
+    int2* row = cnt + (int64_t)t * nchunks;
+    if (threadIdx.x == 0) row[blockIdx.x] = make_int2(total & 0xFFFF, total >> 16);
+    const int blocks = (nodes[c.node].size + kChunk - 1) / kChunk;
+    if (!last_block(&sp->ticket, blocks)) return;
+    int lrun = 0, erun = 0;
+    for (int c0 = 0; c0 < blocks; c0 += NT) {
+        const int i = c0 + threadIdx.x;
+        int2 x = make_int2(0, 0);
+        if (i < blocks) {
+            x.x = __ldcg(&row[c.first + i].x);
+            x.y = __ldcg(&row[c.first + i].y);
         }
-        return lo;
-    };
-    const int c_beg = first_of(s), c_end = first_of(s + 1);
-    int32_t* row = cnt_to_base + (int64_t)t * nchunks;
-    int run = 0;
-    for (int c0 = c_beg; c0 < c_end; c0 += NT) {
-        const int c = c0 + threadIdx.x;
-        const int v = c < c_end ? row[c] : 0;
-        int total;
-        const int pre = block_excl_scan<NT>(v, sh, &total);
-        if (c < c_end) row[c] = run + pre;
-        run += total;
+        int lt, et;
+        const int lp = block_excl_scan<NT>(x.x, sh, &lt);
+        const int ep = block_excl_scan<NT>(x.y, sh, &et);
+        if (i < blocks) row[c.first + i] = make_int2(lrun + lp, erun + ep);
+        lrun += lt;
+        erun += et;
     }
 }
 
@@ -969,25 +990,46 @@ __global__ void __launch_bounds__(NT) big_scatter_kernel(int64_t n, int S, int n
                                                          const uint32_t* __restrict__ keys,
                                                          const int32_t* __restrict__ perm_cur,
                                                          const SelState* __restrict__ st,
-                                                         const int32_t* __restrict__ lbase_arr,
+                                                         const int2* __restrict__ cnt,
                                                          int32_t* perm_nxt, int32_t* node_pos, int32_t* pos_of,
                                                          int32_t* node_of, int id_mode, const int* xb_bad)
 {
-    __shared__ unsigned long long k64[kChunk];
-    __shared__ int sh[33];
+    constexpr int R = kChunk / NT;  // rounds: the slice's keys and ids are loaded up front
+    __shared__ int sh[2 * (NT / 32)];
     const Chunk c = chunks[blockIdx.x];
     const int t = blockIdx.y;
     const SplitNode nd = nodes[c.node];
-    const unsigned long long thr = st[(int64_t)t * S + c.node].thr;
+    const SelState s = st[(int64_t)t * S + c.node];
     const int64_t row = (int64_t)t * n;
-    for (int e = threadIdx.x; e < c.len; e += NT)
-        k64[e] = ((unsigned long long)keys[row + c.start + e] << 32) | (uint32_t)perm_cur[row + c.start + e];
-    __syncthreads();
-    const int32_t lb = lbase_arr[(int64_t)t * nchunks + blockIdx.x];
-    const int32_t before = c.start - nd.off;
-    stable_scatter<NT>(k64, c.len, thr, nd.off + lb, nd.off + nd.size / 2 + (before - lb), nd.childL,
-                       nd.childR, perm_nxt + row, node_pos + row, pos_of + row, node_of + row,
-                       want_id_maps(id_mode, xb_bad), sh);
+    uint32_t kv[R];
+    int32_t id[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int e = r * NT + threadIdx.x;
+        kv[r] = e < c.len ? keys[row + c.start + e] : 0u;
+        id[r] = e < c.len ? perm_cur[row + c.start + e] : 0;
+    }
+    const int2 before = cnt[(int64_t)t * nchunks + blockIdx.x];
+    const bool id_maps = want_id_maps(id_mode, xb_bad);
+    int lb = before.x, eb = before.y;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int e = r * NT + threadIdx.x;
+        const bool live = e < c.len;
+        bool left;
+        const int lefts =
+            split_round<NT>(live && kv[r] < s.prefix, live && kv[r] == s.prefix, s.rank, r, sh, lb, eb, left);
+        if (live) {
+            const int32_t dst = left ? nd.off + lefts : nd.off + nd.size / 2 + (c.start - nd.off + e - lefts);
+            const int32_t child = left ? nd.childL : nd.childR;
+            perm_nxt[row + dst] = id[r];
+            node_pos[row + dst] = child;
+            if (id_maps) {
+                pos_of[row + id[r]] = dst;
+                node_of[row + id[r]] = child;
+            }
+        }
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1040,16 +1082,25 @@ cudaError_t run_partition(const XDesc& x, const TreePlan& P, const DevPlan& dp, 
     int32_t* node_of = ar.take<int32_t>((size_t)T * n);
     int32_t* node_pos = ar.take<int32_t>((size_t)T * n);
     uint32_t* keys = ar.take<uint32_t>((size_t)T * n);
-    float* dirs = ar.take<float>((size_t)T * S_max * d_pad);
+    // the directions of a run of levels at a time: as many levels as 64 MB
+    // (or one level) hold
+    int64_t dir_cap = std::max<int64_t>((int64_t)T * S_max, ((int64_t)64 << 20) / (4 * (int64_t)d_pad));
+    {
+        int64_t all = 0;
+        for (const LevelPlan& L : P.levels) all += (int64_t)T * L.nnodes;
+        dir_cap = std::max<int64_t>(1, std::min(dir_cap, all));
+    }
+    float* dir_buf = ar.take<float>((size_t)dir_cap * d_pad);
+    float* dirs = nullptr;  // of the level
     const int S_big = std::max(P.max_big_nodes, 1);
     SelState* sel = ar.take<SelState>((size_t)T * S_big);
-    uint32_t* ghist = ar.take<uint32_t>((size_t)T * S_big * 256);
-    int32_t* cnt = ar.take<int32_t>((size_t)T * std::max(P.max_chunks, 1));
+    uint32_t* ghist = ar.take<uint32_t>((size_t)T * S_big * kBigBins);
+    int2* cnt = ar.take<int2>((size_t)T * std::max(P.max_chunks, 1));
     uint32_t* rmin = nullptr;
     uint32_t* rmax = nullptr;
     if (lf && lf->C > 0) {
         rmin = ar.take<uint32_t>((size_t)T * S_max);
-        rmax = ar.take<uint32_t>((size_t)T * S_max);
+        rmax = ar.take<uint32_t>((size_t)T * S_max + 1);  // and the flat-node word
     }
     if (!ar.base) return cudaSuccess;  // measuring only
 
@@ -1077,8 +1128,14 @@ cudaError_t run_partition(const XDesc& x, const TreePlan& P, const DevPlan& dp, 
         init_root_nodes_kernel<<<dim3(slices, P.levels[0].nnodes, T), 256, 0, st>>>(n, dp.nodes, node_of, node_pos);
         note_launches(1);
     }
+    // tickets and histograms of the multi-block split: zero between its passes
+    if (P.max_big_nodes > 0) {
+        cudaMemsetAsync(sel, 0, sizeof(SelState) * (size_t)T * S_big, st);
+        cudaMemsetAsync(ghist, 0, sizeof(uint32_t) * (size_t)T * S_big * kBigBins, st);
+    }
     int32_t* cur = perm_a;
     int32_t* nxt = perm_b;
+    int dir_next = 0;  // first level without directions
     for (size_t lvl = 0; lvl < P.levels.size(); ++lvl) {
         const LevelPlan& L = P.levels[lvl];
         const SplitNode* nodes = dp.nodes + L.node_base;
@@ -1086,8 +1143,6 @@ cudaError_t run_partition(const XDesc& x, const TreePlan& P, const DevPlan& dp, 
         const bool learned = lf && lf->Z && (int)lvl < lf->C;
         LevelFeat lv{};
         if (learned) {
-            lv.Z = lf->Z;
-            lv.C = lf->C;
             for (int t = 0; t < T && t0 + t < 32; ++t) lv.ft.f[t] = lf->feat[t0 + t][lvl];
             lv.rmin = rmin;
             lv.rmax = rmax;
@@ -1095,14 +1150,34 @@ cudaError_t run_partition(const XDesc& x, const TreePlan& P, const DevPlan& dp, 
             lv.tau = lf->tau;
             cudaMemsetAsync(rmin, 0xFF, sizeof(uint32_t) * (size_t)T * S, st);
             cudaMemsetAsync(rmax, 0, sizeof(uint32_t) * (size_t)T * S, st);
+            int* any = reinterpret_cast<int*>(rmax + (size_t)T * S_max);
+            cudaMemsetAsync(any, 0, sizeof(int), st);
+            lv.any_flat = any;
             node_feature_range_kernel<<<grid_for((int64_t)T * n, 256, gcap), 256, 0, st>>>(n, T, lf->Z, lf->C, lv.ft,
                                                                                          node_pos, cur, S, rmin,
-                                                                                         rmax);
-            note_launches(1);
+                                                                                         rmax, keys);
+            learned_flat_kernel<<<(int)(((int64_t)T * S + 255) / 256), 256, 0, st>>>(T, S, lv, any);
+            note_launches(2);
         }
-        gen_dirs_kernel<<<grid_for((int64_t)T * S * (d_pad / 4), 256, gcap), 256, 0, st>>>(
-            dirs, T, S, x.d, d_pad, nodes, (uint32_t)lvl, seed, (uint32_t)t0);
-        note_launches(1);
+        if ((int)lvl == dir_next) {
+            DirLevels dl{};
+            dl.first = (uint32_t)lvl;
+            int64_t end = 0;
+            while (dir_next < (int)P.levels.size() && dl.count < kMaxDirLevels &&
+                   end + (int64_t)T * P.levels[dir_next].nnodes <= dir_cap) {
+                const LevelPlan& Q = P.levels[dir_next++];
+                end += (int64_t)T * Q.nnodes;
+                dl.S[dl.count] = Q.nnodes;
+                dl.node_base[dl.count] = Q.node_base;
+                dl.end[dl.count++] = end;
+            }
+            gen_dirs_kernel<<<grid_for(end * (d_pad / 4), 256, gcap), 256, 0, st>>>(dir_buf, x.d, d_pad, dp.nodes, dl,
+                                                                                    seed, (uint32_t)t0);
+            note_launches(1);
+            dirs = dir_buf;
+        } else {
+            dirs += (int64_t)T * P.levels[lvl - 1].nnodes * d_pad;
+        }
         if (pca && pca->on) {
             // principal directions of the nodes' samples, from the random ones
             const cudaError_t e = run_pca_dirs(x, T, S, nodes, cur, d_pad, (uint32_t)lvl, seed, t0, dirs, pca->out,
@@ -1167,17 +1242,16 @@ cudaError_t run_partition(const XDesc& x, const TreePlan& P, const DevPlan& dp, 
         for (int s = 0; s < S; ++s) covered += P.nodes[L.node_base + s].size;
         if (covered < n) cudaMemcpyAsync(nxt, cur, sizeof(int32_t) * (size_t)T * n, cudaMemcpyDeviceToDevice, st);
         if (L.nbig < S) {
-            constexpr int NT = 512;
-            const size_t smem = sizeof(unsigned long long) * (size_t)L.max_small;
-            static bool attr = false;
-            if (!attr) {
-                cudaError_t e = cudaFuncSetAttribute(split_small_kernel<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                     (int)(sizeof(unsigned long long) * kSmallCap));
-                if (e != cudaSuccess) return e;
-                attr = true;
-            }
-            split_small_kernel<NT><<<dim3(S - L.nbig, T), NT, smem, st>>>(n, nodes + L.nbig, keys, cur, nxt, node_pos,
-                                                                         pos_of, node_of, id_mode, x.xb_bad);
+            // threads by the level's largest one-block node
+            const size_t smem = sizeof(uint32_t) * (size_t)L.max_small;
+            const dim3 grid(S - L.nbig, T);
+            auto split = [&](auto kern, int nt) {
+                kern<<<grid, nt, smem, st>>>(n, nodes + L.nbig, keys, cur, nxt, node_pos, pos_of, node_of, id_mode,
+                                             x.xb_bad);
+            };
+            if (L.max_small <= 1024) split(split_small_kernel<128, 8>, 128);
+            else if (L.max_small <= 2048) split(split_small_kernel<256, 9>, 256);
+            else split(split_small_kernel<512, 11>, 512);
             note_launches(1);
         }
         if (L.nbig > 0) {
@@ -1185,22 +1259,16 @@ cudaError_t run_partition(const XDesc& x, const TreePlan& P, const DevPlan& dp, 
             const int SB = L.nbig;
             const Chunk* chunks = dp.chunks + L.chunk_base;
             const int NC = L.nchunks;
-            big_init_kernel<<<(SB * T + 255) / 256, 256, 0, st>>>(SB, T, nodes, sel);
-            note_launches(1);
-            cudaMemsetAsync(ghist, 0, sizeof(uint32_t) * (size_t)T * SB * 256, st);
-            for (int shift = 56; shift >= 0; shift -= 8) {
-                big_hist_kernel<NT><<<dim3(NC, T), NT, 0, st>>>(n, shift, SB, chunks, keys, cur, sel, ghist);
-                note_launches(1);
-                big_pick_kernel<<<dim3(SB, T), 32, 0, st>>>(shift, SB, sel, ghist);
-                note_launches(1);
+            for (int lo = 21, bits = 11; lo >= 0;) {
+                big_hist_kernel<NT><<<dim3(NC, T), NT, 0, st>>>(n, lo, bits, SB, chunks, nodes, keys, sel, ghist);
+                if (lo == 0) break;
+                bits = lo == 21 ? 11 : 10;
+                lo -= bits;
             }
-            big_count_kernel<NT><<<dim3(NC, T), NT, 0, st>>>(n, SB, NC, chunks, keys, cur, sel, cnt);
-            note_launches(1);
-            big_base_kernel<256><<<dim3(SB, T), 256, 0, st>>>(SB, NC, chunks, cnt);
-            note_launches(1);
+            big_count_kernel<NT><<<dim3(NC, T), NT, 0, st>>>(n, SB, NC, chunks, nodes, keys, sel, cnt);
             big_scatter_kernel<NT><<<dim3(NC, T), NT, 0, st>>>(n, SB, NC, chunks, nodes, keys, cur, sel, cnt, nxt,
                                                                node_pos, pos_of, node_of, id_mode, x.xb_bad);
-            note_launches(1);
+            note_launches(5);
         }
         std::swap(cur, nxt);
     }
