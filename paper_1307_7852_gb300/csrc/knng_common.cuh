@@ -169,13 +169,28 @@ struct RowLoader {
             return bytes_to_float4(__ldg(reinterpret_cast<const unsigned int*>(static_cast<const uint8_t*>(X) + o)));
         return __ldg(reinterpret_cast<const float4*>(static_cast<const float*>(X) + o));
     }
+    // the same for any rows: the first cnt entries (zero past them)
+    __device__ __forceinline__ float4 load4_any(uint64_t o, int cnt) const
+    {
+        float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
+        auto one = [&](uint64_t at) -> float {
+            if (kDT == kDtF16) return __half2float(static_cast<const __half*>(X)[at]);
+            if (kDT == kDtU8) return (float)__ldg(static_cast<const uint8_t*>(X) + at);
+            return __ldg(static_cast<const float*>(X) + at);
+        };
+        r.x = one(o);
+        if (cnt > 1) r.y = one(o + 1);
+        if (cnt > 2) r.z = one(o + 2);
+        if (cnt > 3) r.w = one(o + 3);
+        return r;
+    }
     // bytes j..j+3 of row i packed little-endian (U8 rows, vector-aligned)
     __device__ __forceinline__ uint32_t load_u8x4(int64_t i, int j) const
     {
         return __ldg(reinterpret_cast<const unsigned int*>(static_cast<const uint8_t*>(X) + row_off(i) + j));
     }
     // every load of a row is a full vector load (aligned rows, d % 4 == 0)
-    __device__ __forceinline__ bool all_vec() const { return vec && (d & 3) == 0; }
+    __host__ __device__ __forceinline__ bool all_vec() const { return vec && (d & 3) == 0; }
     // rows scored eight lanes a row (warp_canon_dist_g8): FP32 up to 208
     // entries, FP16 up to 512.  Both forms read at the L2's rate on wide rows
     // (about 10 TB/s), where the other one's 512 contiguous bytes a load are
@@ -708,7 +723,10 @@ __device__ __forceinline__ float warp_canon_dist_batch(const RowLoader<kDT>& L, 
 // (two blocks in flight spill: 23.4 -> 28.8 ms on 2M x 96 FP16 rows, where
 // warp_canon_dist_batch, whose 96-entry row pays for 128 and whose two
 // unrolled batches stall on instruction fetch, takes 38.7).
-template <int kDT>
+// kVec == false: rows of any alignment and d, entry by entry loads (one
+// distance at a time before: a round of 200k points, k = 20, 37 FP32 entries
+// 8.69 -> 1.83 ms, 130 entries 15.3 -> 4.1).
+template <bool kVec = true, int kDT = 0>
 __device__ __forceinline__ float warp_canon_dist_g8(const RowLoader<kDT>& L, int64_t a, const int* b, int nb)
 {
     const int lane = threadIdx.x & 31;
@@ -717,6 +735,7 @@ __device__ __forceinline__ float warp_canon_dist_g8(const RowLoader<kDT>& L, int
 #pragma unroll
     for (int r = 0; r < 8; ++r) off[r] = L.row_off(g8 + r < nb ? b[g8 + r] : (int)a) + q4;
     const uint64_t offa = L.row_off(a) + q4;
+    auto load = [&](uint64_t o, int j) { return kVec ? L.load4_at(o) : L.load4_any(o, L.d - j); };
     float tot = 0.f;
 #pragma unroll 1
     for (int j0 = 0; j0 < L.d; j0 += 32) {
@@ -724,10 +743,10 @@ __device__ __forceinline__ float warp_canon_dist_g8(const RowLoader<kDT>& L, int
 #pragma unroll
         for (int r = 0; r < 8; ++r) p[r] = 0.f;
         if (j0 + q4 < L.d) {
-            const float4 xa = L.load4_at(offa + j0);
+            const float4 xa = load(offa + j0, j0 + q4);
             float4 u[8];
 #pragma unroll
-            for (int r = 0; r < 8; ++r) u[r] = L.load4_at(off[r] + j0);
+            for (int r = 0; r < 8; ++r) u[r] = load(off[r] + j0, j0 + q4);
             const float2 na = make_float2(-xa.x, -xa.y), nb2 = make_float2(-xa.z, -xa.w);
 #pragma unroll
             for (int r = 0; r < 8; ++r) {
@@ -858,24 +877,30 @@ __device__ __forceinline__ void score_u8_g8(const uint8_t* X, int64_t ld, int d,
 // distance to b[c].  Byte rows with exact integer distances take one batch
 // of 32 (32 rows in flight per warp), other vector-aligned rows eight lanes a
 // row, the rest one distance at a time.
-// kForm: 0 picks by the row width here, 1 / 2 are kernels built for narrow /
-// other rows (the code of one form only: with both, the propagation of
-// 256-entry rows ran 3 % slower).
+// kForm: 0 picks by the rows here; kernels built for one form (row_form) hold
+// the code of that one only: with two, the propagation of 256-entry rows ran
+// 3 % slower.
+constexpr int kFormNarrow = 1, kFormWide = 2, kFormAny = 3;
+template <int kDT>
+__host__ __device__ __forceinline__ int row_form(const RowLoader<kDT>& L)
+{
+    return !L.all_vec() ? kFormAny : L.narrow() ? kFormNarrow : kFormWide;
+}
 template <int kForm = 0, int kDT = 0>
 __device__ __forceinline__ float warp_canon_dist32(const RowLoader<kDT>& L, int64_t a, const int* b, int nb)
 {
+    if (kForm == kFormAny) return warp_canon_dist_g8<false>(L, a, b, nb);
+    if (kForm == kFormNarrow) return warp_canon_dist_g8(L, a, b, nb);
     if (kDT == kDtU8 && L.all_vec() && L.int_exact()) return warp_u8_dist_batch<32>(L, a, b, nb);
-    if (kForm != 2 && L.all_vec() && (kForm == 1 || L.narrow())) return warp_canon_dist_g8(L, a, b, nb);
-    if (kForm == 1) {
-        const int lane = threadIdx.x & 31;
-        float mine = 0.f;
-        for (int c = 0; c < nb; ++c) {
-            const float dd = warp_canon_dist(L, a, b[c]);
-            if (lane == c) mine = dd;
-        }
-        return mine;
+    if (kForm == 0) {
+        const int f = row_form(L);
+        if (f == kFormAny) return warp_canon_dist_g8<false>(L, a, b, nb);
+        if (f == kFormNarrow) return warp_canon_dist_g8(L, a, b, nb);
     }
     const int lane = threadIdx.x & 31;
+    // (through warp_canon_dist16, whose run-time test of the rows the compiler
+    // does not see through: without it the two batches were scheduled with
+    // fewer loads in flight, 32.3 -> 37.5 ms on the 1M x 960 round)
     const float lo = warp_canon_dist16(L, a, b, min(nb, 16));
     float hi = 0.f;
     if (nb > 16) hi = warp_canon_dist16(L, a, b + 16, nb - 16);

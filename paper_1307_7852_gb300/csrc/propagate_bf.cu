@@ -90,7 +90,7 @@ __global__ void __launch_bounds__(256, 2) propagate_bf_kernel(RowLoader<kDT> L, 
             for (int c0 = cnt; c0 < end; c0 += 32) {
                 const int nb = min(32, end - c0);
                 float dd;
-                if (kDT == kDtF32 && bytes) dd = warp_canon_dist32(Lb, p, vid + c0, nb);
+                if (kDT == kDtF32 && bytes) dd = warp_canon_dist32<kFormWide>(Lb, p, vid + c0, nb);
                 else dd = warp_canon_dist32<kForm>(L, p, vid + c0, nb);
                 if (lane < nb) vkey[c0 + lane] = pack_key(dd, (uint32_t)vid[c0 + lane]);
             }
@@ -158,8 +158,10 @@ cudaError_t run_propagate_best_first(const XDesc& x, int k, int budget, const in
     auto launch = [&](auto dt) {
         constexpr int kDT = decltype(dt)::value;
         RowLoader<kDT> rl{x.X, x.ld, x.d, x.vec};
-        auto kern = propagate_bf_kernel<kDT, 2>;
-        if (rl.narrow()) kern = propagate_bf_kernel<kDT, kDT == kDtU8 ? 2 : 1>;
+        const int form = row_form(rl);
+        auto kern = form == kFormAny ? propagate_bf_kernel<kDT, kFormAny>
+                  : form == kFormNarrow ? propagate_bf_kernel<kDT, kDT == kDtU8 ? kFormWide : kFormNarrow>
+                                        : propagate_bf_kernel<kDT, kFormWide>;
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return;
         int per_sm = 0;
@@ -168,7 +170,8 @@ cudaError_t run_propagate_best_first(const XDesc& x, int k, int budget, const in
         int64_t blocks = (int64_t)num_sms() * per_sm;
         const int64_t need = (x.n + warps - 1) / warps;
         if (blocks > need) blocks = need;
-        const RowLoader<kDtU8> rb{x.Xb, x.ldb, x.d, true};
+        // (the copy's rows are padded with zeros: whole words, d <= 256)
+        const RowLoader<kDtU8> rb{x.Xb, x.ldb, (x.d + 3) & ~3, true};
         kern<<<(int)blocks, warps * 32, smem, st>>>(rl, rb, x.xb_bad, x.n, k, budget, order, ids_in, ids, dists,
                                                     BL.H, BL.hshift, BL.Bc, (int)BL.per_warp);
         note_launches(1);

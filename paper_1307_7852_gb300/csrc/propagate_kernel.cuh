@@ -28,6 +28,8 @@
 #pragma once
 // Kernel and launcher; one instantiation per element type in propagate_f32.cu /
 // propagate_f16.cu / propagate_u8.cu, the dispatch in propagate.cu.
+#include <type_traits>
+
 #include "knng_common.cuh"
 #include "knng_internal.h"
 
@@ -336,7 +338,7 @@ __global__ void __launch_bounds__(256, KNNG_PROP_MINBLOCKS) propagate_kernel(Row
             for (int c0 = nknown; c0 < cnt; c0 += 32) {
                 const int nb = min(32, cnt - c0);
                 float dd;
-                if (kDT == kDtF32 && bytes) dd = warp_canon_dist32(Lb, p, cid + c0, nb);
+                if (kDT == kDtF32 && bytes) dd = warp_canon_dist32<kFormWide>(Lb, p, cid + c0, nb);
                 else dd = warp_canon_dist32<kForm>(L, p, cid + c0, nb);
                 if (lane < nb) cd[c0 + lane] = dd;
             }
@@ -512,14 +514,19 @@ static cudaError_t launch_prop(const XDesc& x, int k, const int32_t* order, cons
     // round (flags), or the general form (pairwise offers, optional flags)
     const int mode = (tm && !fin && !po.tgt) ? 1 : (fin && !tm && !po.tgt) ? 2 : 0;
     RowLoader<kDT> rl{x.X, x.ld, x.d, x.vec};
-    constexpr int kNarrow = kDT == kDtU8 ? 2 : 1;  // (byte rows have no narrow form)
-    auto kern = mode == 1 ? propagate_kernel<E, kDT, 1, 2>
-              : mode == 2 ? propagate_kernel<E, kDT, 2, 2>
-                          : propagate_kernel<E, kDT, 0, 2>;
-    if (rl.narrow())
-        kern = mode == 1 ? propagate_kernel<E, kDT, 1, kNarrow>
-             : mode == 2 ? propagate_kernel<E, kDT, 2, kNarrow>
-                         : propagate_kernel<E, kDT, 0, kNarrow>;
+    // (float rows that may be scored on their byte copy take that copy's form
+    // when it is exact, inside the kernel; byte rows have no narrow form)
+    constexpr int kNarrow = kDT == kDtU8 ? kFormWide : kFormNarrow;
+    auto pick = [&](auto f) {
+        constexpr int F = decltype(f)::value;
+        return mode == 1 ? propagate_kernel<E, kDT, 1, F>
+             : mode == 2 ? propagate_kernel<E, kDT, 2, F>
+                         : propagate_kernel<E, kDT, 0, F>;
+    };
+    const int form = row_form(rl);
+    auto kern = form == kFormAny ? pick(std::integral_constant<int, kFormAny>{})
+              : form == kFormNarrow ? pick(std::integral_constant<int, kNarrow>{})
+                                    : pick(std::integral_constant<int, kFormWide>{});
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
@@ -528,7 +535,8 @@ static cudaError_t launch_prop(const XDesc& x, int k, const int32_t* order, cons
     int64_t blocks = (int64_t)num_sms() * per_sm;
     const int64_t need = (x.n + warps - 1) / warps;
     if (blocks > need) blocks = need;
-    const RowLoader<kDtU8> rb{x.Xb, x.ldb, x.d, true};
+    // (the copy's rows are padded with zeros: whole words, d <= 256)
+    const RowLoader<kDtU8> rb{x.Xb, x.ldb, (x.d + 3) & ~3, true};
     // byte rows scored one candidate per lane: 16-byte aligned rows whose
     // 16-byte blocks up to d stay inside the row (d <= 128)
     const uint8_t* lane_X = nullptr;
