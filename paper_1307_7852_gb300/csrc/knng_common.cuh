@@ -835,7 +835,8 @@ __device__ __forceinline__ float warp_canon_dist16(const RowLoader<kDT>& L, int6
 // candidate, lane l taking bytes 16 (l mod 8) .. + 15 of its row, so one load
 // instruction fetches four whole rows.  load_query_u8 gives each lane its
 // 16 bytes of the query row; score_u8_g8 writes the distances from a to
-// b[0..nb) (nb <= 32) to out[0..nb) (shared memory).
+// b[0..nb) (nb <= 32) to out[0..nb) (shared memory); dist_u8_g8 returns them
+// (lane l < nb: b[l]) for few candidates at a time, four per step.
 __device__ __forceinline__ uint4 load_query_u8(const uint8_t* X, int64_t ld, int64_t a, int d)
 {
     const int c = threadIdx.x & 7;
@@ -871,6 +872,38 @@ __device__ __forceinline__ void score_u8_g8(const uint8_t* X, int64_t ld, int d,
         const int idx = 4 * it + g;
         if (c == 0 && idx < nb) out[idx] = (float)acc;
     }
+}
+
+__device__ __forceinline__ float dist_u8_g8(const uint8_t* X, int64_t ld, int d, uint4 q, const int* b, int nb)
+{
+    const int lane = threadIdx.x & 31;
+    const int c = lane & 7, g = lane >> 3;
+    uint32_t mine = 0u;  // of candidate lane = 4 it + g', from lane 8 g'
+#pragma unroll 1
+    for (int it = 0; 4 * it < nb; it += 2) {
+        uint4 x[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int idx = 4 * (it + h) + g;
+            x[h] = make_uint4(0u, 0u, 0u, 0u);
+            if (idx < nb && 16 * c < d)
+                x[h] = __ldg(reinterpret_cast<const uint4*>(X + (uint64_t)(uint32_t)b[idx] * (uint32_t)ld + 16 * c));
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            uint32_t t, acc = 0u;
+            t = __vabsdiffu4(q.x, x[h].x); acc = __dp4a(t, t, acc);
+            t = __vabsdiffu4(q.y, x[h].y); acc = __dp4a(t, t, acc);
+            t = __vabsdiffu4(q.z, x[h].z); acc = __dp4a(t, t, acc);
+            t = __vabsdiffu4(q.w, x[h].w); acc = __dp4a(t, t, acc);
+            acc += __shfl_xor_sync(KNNG_FULL_MASK, acc, 4);
+            acc += __shfl_xor_sync(KNNG_FULL_MASK, acc, 2);
+            acc += __shfl_xor_sync(KNNG_FULL_MASK, acc, 1);
+            const uint32_t v = __shfl_sync(KNNG_FULL_MASK, acc, 8 * (lane & 3));
+            if ((lane >> 2) == it + h) mine = v;
+        }
+    }
+    return (float)mine;
 }
 
 // Canonical distances from a to b[0..nb) (nb <= 32): lane c < nb returns the
