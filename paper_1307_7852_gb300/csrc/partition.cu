@@ -400,10 +400,99 @@ __device__ __forceinline__ void project_body(const Loader& L, int64_t n, int T, 
     }
 }
 
+// The same for rows of at most 256 entries.  The first three pairwise rounds
+// halve the set of trees a lane sums (it keeps half of its sums and receives
+// its partner's copy of them: the same additions, 9 shuffles instead of 40),
+// so tree t0 + u ends in the lanes 4u .. 4u + 3; lane 4u looks the point's node
+// and position up and writes the key.
+// What bounds it: the chain of node, row and direction loads of a chunk or
+// two, so the next point's nodes and positions are loaded while this one is
+// projected.  1M points, 6 trees, 13 levels, project_body -> this: 64 entries
+// 7.87 -> 6.84 ms, 128 8.06 -> 7.05, 256 10.5 -> 10.1; at 960 entries (8 trees,
+// 11 levels), where the directions' 11 TB/s from L2 are the bound, its
+// registers cost more than it gives: 30.0 -> 34.0.
+template <bool kLearned, class Loader>
+__device__ __forceinline__ void project_body_short(const Loader& L, int64_t n, int T, const float* __restrict__ dirs,
+                                             int S, int d_pad, const int32_t* __restrict__ node_of,
+                                             const int32_t* __restrict__ pos_of, uint32_t* __restrict__ keys,
+                                             const LevelFeat& lv)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    // lane 4u: node and position of point i in tree t0 + u (-1: none)
+    auto look_up = [&](int64_t i, int t0, int& s, int& pos) {
+        const int tl = t0 + (lane >> 2);
+        s = -1;
+        pos = 0;
+        if ((lane & 3) == 0 && tl < T && i < n) {
+            s = node_of[(int64_t)tl * n + i];
+            pos = pos_of[(int64_t)tl * n + i];
+        }
+    };
+    int next_s, next_pos;
+    look_up(warp, 0, next_s, next_pos);
+    for (int64_t i = warp; i < n; i += nwarps) {
+        // the warp's next row streams into L2 while this one is projected: the
+        // chunk loads below then wait on L2, not on DRAM
+        if (i + nwarps < n) L.prefetch_l2(i + nwarps, lane);
+        int my_s = next_s, my_pos = next_pos;
+        look_up(i + nwarps, 0, next_s, next_pos);
+        for (int t0 = 0; t0 < T; t0 += 8) {
+            const int tl = t0 + (lane >> 2);
+            if (t0 > 0) look_up(i, t0, my_s, my_pos);
+            // learned levels: a node that splits on its learned feature has
+            // its keys and needs no projection
+            if (kLearned && my_s >= 0 && lv.varies(tl, (int64_t)tl * S + my_s)) my_s = -1;
+            if (__ballot_sync(KNNG_FULL_MASK, my_s >= 0) == 0) continue;
+            int sv[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) sv[u] = __shfl_sync(KNNG_FULL_MASK, my_s, 4 * u);
+            float acc[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) acc[u] = 0.0f;
+            for (int j = 4 * lane; j < L.d; j += 128) {
+                const float4 x = L.load4(i, j);
+                const bool full = j + 3 < L.d;
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    if (sv[u] < 0) continue;
+                    const float4 a = *reinterpret_cast<const float4*>(
+                        dirs + ((int64_t)(t0 + u) * S + sv[u]) * d_pad + j);
+                    if (full) {
+                        acc[u] = fmaf(x.x, a.x, acc[u]);
+                        acc[u] = fmaf(x.y, a.y, acc[u]);
+                        acc[u] = fmaf(x.z, a.z, acc[u]);
+                        acc[u] = fmaf(x.w, a.w, acc[u]);
+                    } else {
+                        acc[u] = fmaf(x.x, a.x, acc[u]);
+                        if (j + 1 < L.d) acc[u] = fmaf(x.y, a.y, acc[u]);
+                        if (j + 2 < L.d) acc[u] = fmaf(x.z, a.z, acc[u]);
+                    }
+                }
+            }
+#pragma unroll
+            for (int o = 16, h = 4; o >= 4; o >>= 1, h >>= 1) {
+                const bool hi = (lane & o) != 0;
+#pragma unroll
+                for (int u = 0; u < h; ++u) {
+                    const float send = hi ? acc[u] : acc[u + h];
+                    const float keep = hi ? acc[u + h] : acc[u];
+                    acc[u] = keep + __shfl_xor_sync(KNNG_FULL_MASK, send, o);
+                }
+            }
+            acc[0] += __shfl_xor_sync(KNNG_FULL_MASK, acc[0], 2);
+            acc[0] += __shfl_xor_sync(KNNG_FULL_MASK, acc[0], 1);
+            if (my_s >= 0) keys[(int64_t)tl * n + my_pos] = ord_key(acc[0]);
+        }
+    }
+}
+
 // Float rows whose byte copy is exact (*xb_bad == 0, see XDesc) are read from
 // the copy: the same float values, a quarter of the bytes.  With
 // bytes_elsewhere set, such a build is left to project_bytes_kernel.
-template <int kDT, bool kLearned>
+// kShort: rows of at most 256 entries.
+template <int kDT, bool kLearned, bool kShort>
 __global__ void __launch_bounds__(256) project_kernel(RowLoader<kDT> L, RowLoader<kDtU8> Lb,
                                                       const int* __restrict__ xb_bad, bool bytes_elsewhere,
                                                       int64_t n, int T, const float* __restrict__ dirs, int S,
@@ -415,11 +504,13 @@ __global__ void __launch_bounds__(256) project_kernel(RowLoader<kDT> L, RowLoade
     if constexpr (kDT == kDtF32) {
         if (xb_bad && *xb_bad == 0) {
             if (bytes_elsewhere) return;
-            project_body<kLearned>(Lb, n, T, dirs, S, d_pad, node_of, pos_of, keys, lv);
+            if (kShort) project_body_short<kLearned>(Lb, n, T, dirs, S, d_pad, node_of, pos_of, keys, lv);
+            else project_body<kLearned>(Lb, n, T, dirs, S, d_pad, node_of, pos_of, keys, lv);
             return;
         }
     }
-    project_body<kLearned>(L, n, T, dirs, S, d_pad, node_of, pos_of, keys, lv);
+    if (kShort) project_body_short<kLearned>(L, n, T, dirs, S, d_pad, node_of, pos_of, keys, lv);
+    else project_body<kLearned>(L, n, T, dirs, S, d_pad, node_of, pos_of, keys, lv);
 }
 
 // Exact floats of the four bytes of w: the byte permute assembles 2^23 + b
@@ -1216,12 +1307,12 @@ cudaError_t run_partition(const XDesc& x, const TreePlan& P, const DevPlan& dp, 
                 constexpr int kDT = decltype(dt)::value;
                 RowLoader<kDT> rl{x.X, x.ld, x.d, x.vec};
                 const RowLoader<kDtU8> rb{x.Xb, x.ldb, x.d, true};
-                if (learned)
-                    project_kernel<kDT, true><<<pgrid, 256, 0, st>>>(rl, rb, x.xb_bad, copy_nm, n, T, dirs, S, d_pad,
-                                                                     node_of, pos_of, keys, lv);
-                else
-                    project_kernel<kDT, false><<<pgrid, 256, 0, st>>>(rl, rb, x.xb_bad, copy_nm, n, T, dirs, S, d_pad,
-                                                                      node_of, pos_of, keys, lv);
+                auto go = [&](auto kern) {
+                    kern<<<pgrid, 256, 0, st>>>(rl, rb, x.xb_bad, copy_nm, n, T, dirs, S, d_pad, node_of, pos_of, keys,
+                                                lv);
+                };
+                if (x.d <= 256) go(learned ? project_kernel<kDT, true, true> : project_kernel<kDT, false, true>);
+                else go(learned ? project_kernel<kDT, true, false> : project_kernel<kDT, false, false>);
             };
             if (x.dtype == kDtF16) project(std::integral_constant<int, kDtF16>{});
             else if (x.dtype == kDtU8) project(std::integral_constant<int, kDtU8>{});
