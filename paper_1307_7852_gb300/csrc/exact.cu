@@ -297,9 +297,10 @@ __host__ __device__ __forceinline__ int64_t tile_begin(int64_t total, int G, int
 // 128-byte swizzled K slices of 64 entries; the queries' slices stay in
 // shared memory over a run when they fit), warp 1 issues the MMAs into two
 // 256-column accumulators, warps 2..9 read them back: a thread has one query
-// and 128 of the tile's rows.  The tensor cores take 1,024 cycles for a tile
-// of 128 entries a row and the eight warps about 850 for its minima, so the
-// two overlap at nearly full rate of either.
+// and 128 of the tile's rows.  A tile of 128 entries a row is 1,024 cycles of
+// tensor work and about as much of the eight warps' minima, so the two
+// overlap; 10,000 queries of 1M x 128 take 3.3 ms for the minima and 4.0 ms
+// for the lists (770 and 640 TFLOP/s).
 //  kList == false: minima over 32 groups per thread, written per CTA and
 //   query tile (slot c + rt of CTA c) to mins[slot][128][64].
 //  kList == true: rows with |x^|^2 - 2 q^.x^ <= thr[query] are appended to
@@ -576,13 +577,11 @@ __global__ void __launch_bounds__(256) exact_bound_kernel(int64_t n, int d, int 
         while (c0 > 0 && tile_begin(total, G, c0) > first) --c0;
         while (c1 + 1 < G && tile_begin(total, G, c1 + 1) <= last) ++c1;
         while (c1 > 0 && tile_begin(total, G, c1) > last) --c1;
-        // (a CTA in between without tiles has no minima)
+        // (G <= total: every CTA has tiles)
         const int cnt = (c1 - c0 + 1) * 64;
+        const float* mrow = mins + (((int64_t)c0 + rt) * kTileM + lr) * 64;
         auto key = [&](int i) -> uint64_t {
-            const int c = c0 + (i >> 6);
-            const bool has = tile_begin(total, G, c) < tile_begin(total, G, c + 1);
-            const float v = has ? mins[(((int64_t)c + rt) * kTileM + lr) * 64 + (i & 63)] : kInf;
-            return pack_key(v, (uint32_t)i);
+            return pack_key(mrow[(int64_t)(i >> 6) * (kTileM * 64) + (i & 63)], (uint32_t)i);
         };
         float vk = kInf;
         if (k + 1 <= cnt) {
@@ -705,11 +704,11 @@ static bool exact_rows_map(CUtensorMap* map, void* base, int dq, int64_t rows, i
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// The filtered form pays once the pairs outweigh its six launches and the
-// bfloat16 copy: exact_knn_kernel takes about 2 us per 32 rows whatever the
-// number of queries (up to eight per SM), 130 us at 2,048 rows, the filtered
-// form about 50 us there.  n below 2^31 - 256: row numbers of a tile stay in
-// an int.
+// The filtered form from 2,048 rows on: exact_knn_kernel streams all rows per
+// block, 0.51 ms at 2,048 x 128 for 10 or 1,000 queries and 3.8 ms at 16,384,
+// the filtered form 0.09 / 0.12 ms and 0.15 / 0.19 ms; smaller sets keep the
+// form that needs no scratch.  n below 2^31 - 256: row numbers of a tile stay
+// in an int.
 bool exact_tc_ok(const XDesc& x, int nq)
 {
     return x.n >= 2048 && x.n < ((int64_t)1 << 31) - kTileN && nq > 0;
@@ -763,16 +762,17 @@ cudaError_t run_exact_knn_tc(const XDesc& x, const int32_t* queries, int nq, int
         const int cq = std::min(nq - q0, kBatchQ);
         const int RT = (cq + kTileM - 1) / kTileM, rows = RT * kTileM;
         const int64_t total = (int64_t)RT * CT;
+        const int Gb = (int)std::min<int64_t>(G, total);  // no CTA without a tile
         const int32_t* qs = queries + q0;
         int32_t* oi = ids + (int64_t)q0 * k;
         float* od = dists + (int64_t)q0 * k;
         exact_gather_kernel<<<(int)std::min<int64_t>(((int64_t)rows * (dq / 8) + 255) / 256, (int64_t)G * 8), 256, 0, st>>>(
             reinterpret_cast<const uint4*>(Xq), x.n, dq / 8, qs, cq, rows, reinterpret_cast<uint4*>(Aq));
-        exact_gram_kernel<false><<<G, kGramThreads, smem, st>>>(amap, bmap, nK, RT, CT, a_stays, nrm, mins, nullptr,
+        exact_gram_kernel<false><<<Gb, kGramThreads, smem, st>>>(amap, bmap, nK, RT, CT, a_stays, nrm, mins, nullptr,
                                                                 nullptr, nullptr, err);
-        exact_bound_kernel<<<(rows + 7) / 8, 256, 0, st>>>(x.n, x.d, k, qs, cq, rows, G, CT, total, mins, nrm, xerr,
+        exact_bound_kernel<<<(rows + 7) / 8, 256, 0, st>>>(x.n, x.d, k, qs, cq, rows, Gb, CT, total, mins, nrm, xerr,
                                                            stats, thr, counts, need);
-        exact_gram_kernel<true><<<G, kGramThreads, smem, st>>>(amap, bmap, nK, RT, CT, a_stays, nrm, nullptr, thr,
+        exact_gram_kernel<true><<<Gb, kGramThreads, smem, st>>>(amap, bmap, nK, RT, CT, a_stays, nrm, nullptr, thr,
                                                                counts, lists, err);
         note_launches(4);
         typed([&](auto rl) {

@@ -28,6 +28,10 @@
 // (FP16, bytes, unaligned) are loaded, widened and stored.
 // Leaves that are exact in reduced precision (their lists are final) are
 // skipped by a flag the leaf kernel writes.
+// 1M x 960, 8 trees, k' = 20: 24.7 -> 19.8 ms with the rows in order of their
+// pairs, slots instead of searches, candidates read as 16-byte groups and a
+// third slice; 300k x 384, 6 trees, k' = 40: 9.9 -> 6.2 ms.  (Rolled, sums in
+// shared memory, at k' = 20: 28.4 ms.)
 #include <algorithm>
 #include <type_traits>
 

@@ -499,7 +499,10 @@ __global__ void __launch_bounds__(kTcThreads, PER == 16 ? 1 : 2) leaf_tc_kernel(
     // final lists; the others hand over the selected columns.  Rows whose
     // lists overflow, rows with equal values at the cut, and all rows when
     // more than kListWant candidates (32 of an exact leaf) are wanted take
-    // the warp-per-row path below.
+    // the warp-per-row path below.  (Before, lists of at most 32 a row and no
+    // cut: 200k x 200, 5 trees, k' = 32 took that path for most rows, 5.03 ms
+    // against 0.68 now; sift1m's exact leaves, with packed distances and
+    // predicated list stores, 5.45 -> 3.87.)
     if (!abort_flag) {
         const int quad = w & 3, half = w >> 2;
         const int lr = 32 * quad + lane;

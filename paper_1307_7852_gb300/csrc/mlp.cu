@@ -43,8 +43,8 @@ namespace knng {
 // network's 16 or 32 outputs, where a 64-wide tile would be mostly padding.
 // The weight gradients contract over the batch (K = 8192 rows of a
 // 4,096-edge batch against 256 x 96 outputs): without the K slices 8 blocks
-// did the whole contraction (2.1 ms each of the two on GB300; 11 us with
-// slices over about two blocks per SM).
+// did the whole contraction (4.2 ms for the two; 23 + 11 us with slices over
+// about two blocks per SM, and 7 us to add them up).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ float gelu_f(float a)
 {
@@ -213,7 +213,7 @@ __global__ void sample_batch_kernel(RowLoader<kDT> L, int64_t n, const int32_t* 
 // ---------------------------------------------------------------------------
 // Loss and dL/dZ through the batch statistics.  Z: N x C rows, N = 2B.
 // Four passes over blocks of kLossRows rows (one block did it all before:
-// 0.7 ms of an 8192 x 16 batch, now 12 us): column sums; centred second
+// 0.70 ms of an 8192 x 16 batch, now 56 us in all): column sums; centred second
 // moments and the pairs' differences; the statistics and the loss (one
 // block, sums of the row blocks in FP64); the gradient.
 //   K = corr, S = (z - mean) / sqrt(var + eps), dS = (2/N) S G with
