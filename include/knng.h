@@ -131,14 +131,15 @@ const char* knng_last_error(const knng_handle* h);
  * of those calls are then invalid); the flag is cleared. */
 int knng_sync(knng_handle* h, void* stream);
 
-/* Limit, in SM clock cycles, of the tensor-core leaf kernel's waits for its
- * TMA copies and for the MMAs to release a pipeline stage, for later calls
- * on h (0, the default: 2e9 cycles, about one second).  A CTA whose wait
- * runs out records KNNG_ERR_TIMEOUT for knng_sync, waits (under the one-second
- * limit) for the copies and MMAs it started, frees its tensor memory and
- * returns; the context stays usable.  A small limit makes waits on copies
- * that do complete give up -- a way to exercise that path.  cycles < 0:
- * KNNG_ERR_INVALID_ARG.  No counterpart in the paper. */
+/* Limit, in SM clock cycles, of the waits of the tensor-core leaf kernel and
+ * of the tensor-core passes of knng_exact_knn for their TMA copies and MMAs,
+ * for later calls on h (0, the default: 2e9 cycles, about one second).  A CTA
+ * whose wait runs out records KNNG_ERR_TIMEOUT for knng_sync, waits (under
+ * the one-second limit) for the copies and MMAs it started, frees its tensor
+ * memory and returns; the context stays usable (knng_exact_knn then answers
+ * with its direct form, so its lists stay valid).  A small limit makes waits
+ * on copies that do complete give up -- a way to exercise that path.
+ * cycles < 0: KNNG_ERR_INVALID_ARG.  No counterpart in the paper. */
 int knng_set_wait_limit(knng_handle* h, int64_t cycles);
 
 /* Counters of what the first-order propagation rounds read (Sec. 3.2;

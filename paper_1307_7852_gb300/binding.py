@@ -428,8 +428,9 @@ def knng_set_stage_events(events, h: Handle):
 
 
 def knng_set_wait_limit(cycles: int, h: Handle):
-    """Limit (SM cycles, 0 = about one second) of the tensor-core leaf
-    kernel's pipeline waits for later calls on h."""
+    """Limit (SM cycles, 0 = about one second) of the pipeline waits of the
+    tensor-core leaf kernel and of the exact k-NN's tensor-core passes, for
+    later calls on h."""
     h.check(lib().knng_set_wait_limit(h.ptr, int(cycles)), "knng_set_wait_limit")
 
 

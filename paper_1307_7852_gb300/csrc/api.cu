@@ -76,7 +76,7 @@ struct knng_handle {
     char* exact_ws = nullptr;
     size_t exact_ws_size = 0;
     cudaEvent_t exact_done = nullptr;
-    long long wait_cycles = 0;   // limit of the leaf kernel's pipeline waits (0: about 1 s)
+    long long wait_cycles = 0;   // limit of the leaf and exact kernels' pipeline waits (0: about 1 s)
     unsigned long long* prop_stats = nullptr;  // caller's read counters, 2 per round
     int prop_stats_rounds = 0;
 };
@@ -867,7 +867,7 @@ int knng_exact_knn(knng_handle* h, const void* X, int32_t dtype, int64_t n, int3
     if (exact_tc_ok(x, (int)nq) && exact_scratch(h, x, (int)nq, k, st)) {
         Arena a;
         a.base = h->exact_ws;
-        e = run_exact_knn_tc(x, queries, (int)nq, k, ids, dists, h->dev_err, a, st);
+        e = run_exact_knn_tc(x, queries, (int)nq, k, ids, dists, h->dev_err, a, st, h->wait_cycles);
         const cudaError_t e2 = cudaEventRecord(h->exact_done, st);
         if (e == cudaSuccess) e = e2;
     } else {

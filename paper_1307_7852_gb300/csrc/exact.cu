@@ -28,10 +28,10 @@
 //      (a few tens on descriptor data);
 //   5. exact_rescore_kernel: canonical distances of the listed rows, the k
 //      best by (distance, id).
-// Queries whose list overflows, and all of them when a row is not finite,
-// are answered by exact_knn_kernel.  10,000 queries of 1,000,000 x 128
-// rows, k = 20: 788 ms with exact_knn_kernel alone (seven shuffles per pair
-// and 128 entries), 7.6 ms filtered.
+// Queries whose list overflows, and all of them when a row is not finite or a
+// bounded wait gave up, are answered by exact_knn_kernel.
+// 10,000 queries of 1,000,000 x 128 rows, k = 20: 788 ms with exact_knn_kernel
+// alone (seven shuffles per pair and 128 entries), 7.6 ms filtered.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>
@@ -201,7 +201,8 @@ constexpr int kBatchQ = 16384;      // queries per batch: fewer row tiles than S
                                     // every query's rows are split over at least two CTAs
 constexpr int kListMax = 1024;      // listed rows per query
 constexpr int kRescoreWarps = 4;
-constexpr long long kExactWait = 2000000000LL;  // ~1 s at GB300 clocks
+constexpr long long kExactWait = 2000000000LL;  // ~1 s at GB300 clocks: the default limit of the
+                                                // waits, and the limit of the drains
 
 // Largest |x - x^| and |x^|^2 over the rows (as order-preserving words of
 // non-negative floats) and whether a row is not finite.
@@ -309,7 +310,7 @@ template <bool kList>
 __global__ void __launch_bounds__(kGramThreads, 1) exact_gram_kernel(
     const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUtensorMap bmap, int nK, int RT, int CT,
     bool a_stays, const float* __restrict__ nrm, float* __restrict__ mins, const float* __restrict__ thr,
-    int* __restrict__ counts, int32_t* __restrict__ lists, int* err)
+    int* __restrict__ counts, int32_t* __restrict__ lists, long long limit, int* err)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     unsigned char* base = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -352,7 +353,7 @@ __global__ void __launch_bounds__(kGramThreads, 1) exact_gram_kernel(
     // a bounded wait that also ends when another warp gave up
     auto wait = [&](uint64_t* bar, uint32_t parity) -> bool {
         if (abort_flag) return false;
-        if (tc::mbar_wait(bar, parity, kExactWait)) return true;
+        if (tc::mbar_wait(bar, parity, limit)) return true;
         give_up();
         return false;
     };
@@ -396,20 +397,19 @@ __global__ void __launch_bounds__(kGramThreads, 1) exact_gram_kernel(
                     ++rt;
                 }
             }
-            if (!ok) {
-                // the copies in flight land before the CTA ends (bounded)
-                for (int64_t q = it > kGramStages ? it - kGramStages : 0; q < it; ++q)
-                    tc::mbar_wait(&full[q % kGramStages], (uint32_t)(q / kGramStages) & 1u, kExactWait);
-                for (uint32_t q = ntimes > 2 ? ntimes - 2 : 0; q < ntimes; ++q)
-                    tc::mbar_wait(&nfull[q & 1u], (q >> 1) & 1u, kExactWait);
-                if (atimes) tc::mbar_wait(&afull, (atimes - 1) & 1u, kExactWait);
-            }
+            // every copy has landed before the CTA ends (bounded), also when
+            // this warp issued all of its own and another one gave up on them
+            for (int64_t q = it > kGramStages ? it - kGramStages : 0; q < it; ++q)
+                tc::mbar_wait(&full[q % kGramStages], (uint32_t)(q / kGramStages) & 1u, kExactWait);
+            for (uint32_t q = ntimes > 2 ? ntimes - 2 : 0; q < ntimes; ++q)
+                tc::mbar_wait(&nfull[q & 1u], (q >> 1) & 1u, kExactWait);
+            if (atimes) tc::mbar_wait(&afull, (atimes - 1) & 1u, kExactWait);
         }
         __syncwarp();
     } else if (w == 1) {
         if (lane == 0) {
             const uint32_t idesc = tc::make_idesc(1u, kTileM, kTileN);
-            int64_t it = 0;
+            int64_t it = 0, done = 0;  // K slices, whole tiles
             int rt_cur = -1;
             uint32_t atimes = 0;
             bool ok = true;
@@ -436,17 +436,21 @@ __global__ void __launch_bounds__(kGramThreads, 1) exact_gram_kernel(
                                     tc::sw128_desc(sb + kk * 32), idesc, (kc | kk) ? 1u : 0u);
                     tc::mma_commit(&empty[s]);
                 }
-                if (ok) tc::mma_commit(&tfull[b]);
+                if (ok) {
+                    tc::mma_commit(&tfull[b]);
+                    ++done;
+                }
                 if (++ct == CT) {
                     ct = 0;
                     ++rt;
                 }
             }
-            if (!ok && it > 0) {
-                // the MMAs in flight end before the accumulators are freed
-                const int64_t q = it - 1;
-                tc::mbar_wait(&empty[q % kGramStages], (uint32_t)(q / kGramStages) & 1u, kExactWait);
-            }
+            // the MMAs have ended (and signalled) before the accumulators are
+            // freed and the CTA ends, also when all were issued and a warp
+            // that reads them gave up
+            if (it > 0)
+                tc::mbar_wait(&empty[(it - 1) % kGramStages], (uint32_t)((it - 1) / kGramStages) & 1u, kExactWait);
+            if (done > 0) tc::mbar_wait(&tfull[(done - 1) & 1], (uint32_t)((done - 1) >> 1) & 1u, kExactWait);
         }
         __syncwarp();
     } else {
@@ -620,12 +624,13 @@ __global__ void __launch_bounds__(256) exact_bound_kernel(int64_t n, int d, int 
 }
 
 // One warp per query: canonical distances of its listed rows, the k best by
-// (distance, id).  Marks overflowing queries for exact_knn_kernel.
+// (distance, id).  Marks queries whose list overflowed, and all of them once a
+// bounded wait gave up, for exact_knn_kernel.
 template <int kDT>
 __global__ void __launch_bounds__(kRescoreWarps * 32) exact_rescore_kernel(
     RowLoader<kDT> L, int64_t n, const int32_t* __restrict__ queries, int nq, int k, const int* __restrict__ counts,
-    const int32_t* __restrict__ lists, uint8_t* __restrict__ need, int32_t* __restrict__ out_ids,
-    float* __restrict__ out_d)
+    const int32_t* __restrict__ lists, uint8_t* __restrict__ need, const int* __restrict__ err,
+    int32_t* __restrict__ out_ids, float* __restrict__ out_d)
 {
     __shared__ uint64_t buf_all[kRescoreWarps][kListMax];
     __shared__ uint32_t hist_all[kRescoreWarps][256];
@@ -636,7 +641,8 @@ __global__ void __launch_bounds__(kRescoreWarps * 32) exact_rescore_kernel(
     if (qi >= nq) return;
     if (need[qi]) return;
     const int cnt = counts[qi];
-    if (cnt > kListMax) {
+    // (a wait that gave up leaves rows unlisted: the direct kernel answers)
+    if (cnt > kListMax || *err != 0) {
         if (lane == 0) need[qi] = 1;
         return;
     }
@@ -714,11 +720,13 @@ bool exact_tc_ok(const XDesc& x, int nq)
     return x.n >= 2048 && x.n < ((int64_t)1 << 31) - kTileN && nq > 0;
 }
 
-// Scratch from ar (measured with ar.base == nullptr).  *err: word set when a
-// bounded wait gave up.
+// Scratch from ar (measured with ar.base == nullptr).  wait_cycles: limit of
+// the tensor-core passes' waits (0: about one second); *err: word set when one
+// gave up (the direct kernel then answers the queries).
 cudaError_t run_exact_knn_tc(const XDesc& x, const int32_t* queries, int nq, int k, int32_t* ids, float* dists,
-                             int* err, Arena& ar, cudaStream_t st)
+                             int* err, Arena& ar, cudaStream_t st, long long wait_cycles)
 {
+    const long long limit = wait_cycles > 0 ? wait_cycles : kExactWait;
     const int dq = (x.d + 63) / 64 * 64, nK = dq / 64;
     const int CT = (int)((x.n + kTileN - 1) / kTileN);
     const int64_t n_pad = (int64_t)CT * kTileN;
@@ -769,15 +777,15 @@ cudaError_t run_exact_knn_tc(const XDesc& x, const int32_t* queries, int nq, int
         exact_gather_kernel<<<(int)std::min<int64_t>(((int64_t)rows * (dq / 8) + 255) / 256, (int64_t)G * 8), 256, 0, st>>>(
             reinterpret_cast<const uint4*>(Xq), x.n, dq / 8, qs, cq, rows, reinterpret_cast<uint4*>(Aq));
         exact_gram_kernel<false><<<Gb, kGramThreads, smem, st>>>(amap, bmap, nK, RT, CT, a_stays, nrm, mins, nullptr,
-                                                                nullptr, nullptr, err);
+                                                                nullptr, nullptr, limit, err);
         exact_bound_kernel<<<(rows + 7) / 8, 256, 0, st>>>(x.n, x.d, k, qs, cq, rows, Gb, CT, total, mins, nrm, xerr,
                                                            stats, thr, counts, need);
         exact_gram_kernel<true><<<Gb, kGramThreads, smem, st>>>(amap, bmap, nK, RT, CT, a_stays, nrm, nullptr, thr,
-                                                               counts, lists, err);
+                                                               counts, lists, limit, err);
         note_launches(4);
         typed([&](auto rl) {
             exact_rescore_kernel<<<(cq + kRescoreWarps - 1) / kRescoreWarps, kRescoreWarps * 32, 0, st>>>(
-                rl, x.n, qs, cq, k, counts, lists, need, oi, od);
+                rl, x.n, qs, cq, k, counts, lists, need, err, oi, od);
             note_launches(1);
         });
         e = run_exact_knn(x, qs, cq, k, oi, od, st, need);

@@ -267,7 +267,7 @@ cudaError_t run_exact_knn(const XDesc& x, const int32_t* queries, int nq, int k,
 // The same lists with the pairs filtered on the tensor cores (exact.cu).
 bool exact_tc_ok(const XDesc& x, int nq);
 cudaError_t run_exact_knn_tc(const XDesc& x, const int32_t* queries, int nq, int k, int32_t* ids, float* dists,
-                             int* err, Arena& ar, cudaStream_t st);
+                             int* err, Arena& ar, cudaStream_t st, long long wait_cycles = 0);
 
 // One set of a batched build, as seen by the output scatter.
 struct BatchSet {
