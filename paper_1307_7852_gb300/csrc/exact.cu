@@ -254,8 +254,9 @@ __global__ void __launch_bounds__(256) exact_quant_kernel(RowLoader<kDT> L, int6
             s += __shfl_xor_sync(KNNG_FULL_MASK, s, q);
             e += __shfl_xor_sync(KNNG_FULL_MASK, e, q);
         }
-        // (rounded up: the sum's relative error is below (d / 32 + 8) 2^-24)
-        e = sqrtf(e) * 1.0001f;
+        // (rounded up: the sum's relative error is below (d / 32 + 8) 2^-24,
+        // and squares that underflow lose d 2^-149 <= 2^-138 in all)
+        e = sqrtf(e) * 1.0001f + 0x1p-69f;
         if (lane == 0) {
             nrm[r] = s;
             err[r] = e;
@@ -605,8 +606,11 @@ __global__ void __launch_bounds__(256) exact_bound_kernel(int64_t n, int d, int 
             // error of D^: each of the d additions of a product errs by at
             // most 2^-22 of |q^| |x^| <= (|q^|^2 + |x^|^2) / 2; the norms and
             // the combination add less.  Twice that, for the roundings of
-            // this bound itself.
-            const float e = (float)(d + 16) * 0x1p-20f * (ni + ymax);
+            // this bound itself.  Below the normal range the errors are
+            // absolute: 2^-126 for a product or a partial sum flushed to zero
+            // (twice, for the factor 2), 2^-149 for a rounding of the norms or
+            // of the canonical distances; 2^-122 an entry covers them twice.
+            const float e = (float)(d + 16) * (0x1p-20f * (ni + ymax) + 0x1p-122f);
             const float s = (err[q] + __uint_as_float(stats->max_err)) * 1.0001f;
             const float u = sqrtf(fmaxf(ni + vk, 0.f) + e) * 1.0001f + 2.f * s;
             lim = (u * u * 1.0001f + e) - ni;
