@@ -14,7 +14,7 @@
 // The filtered form (run_exact_knn_tc) scores the pairs on the tensor cores
 // and computes the canonical distance only of those that can be listed:
 //   1. x^ = bfloat16(x) of every row, |x^|^2 and the distance |x - x^|;
-//   2. exact_gram_kernel<false>: D^ = |q^|^2 + |x^|^2 - 2 q^.x^ of every
+//   2. exact_gram_kernel (minima): D^ = |q^|^2 + |x^|^2 - 2 q^.x^ of every
 //      pair (tcgen05, FP32 accumulation), reduced to minima over 64 groups of
 //      rows per query and CTA;
 //   3. exact_bound_kernel: the (k+1)-th smallest minimum is at least the
@@ -23,7 +23,7 @@
 //      U = sqrt(D^ + e) + s of the query, so a row of the answer has
 //      D^ <= (U + s)^2 + e (with the relative error of the canonical
 //      distance on top);
-//   4. exact_gram_kernel<true>: the same products again (cheaper than
+//   4. exact_gram_kernel (lists): the same products again (cheaper than
 //      storing n values per query), rows up to that bound listed per query
 //      (a few tens on descriptor data);
 //   5. exact_rescore_kernel: canonical distances of the listed rows, the k
@@ -307,7 +307,8 @@ __host__ __device__ __forceinline__ int64_t tile_begin(int64_t total, int G, int
 //   query tile (slot c + rt of CTA c) to mins[slot][128][64].
 //  kList == true: rows with |x^|^2 - 2 q^.x^ <= thr[query] are appended to
 //   the query's list.
-template <bool kList>
+// kPoll: the waits poll without suspending (limits too short for try_wait).
+template <bool kList, bool kPoll>
 __global__ void __launch_bounds__(kGramThreads, 1) exact_gram_kernel(
     const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUtensorMap bmap, int nK, int RT, int CT,
     bool a_stays, const float* __restrict__ nrm, float* __restrict__ mins, const float* __restrict__ thr,
@@ -354,7 +355,17 @@ __global__ void __launch_bounds__(kGramThreads, 1) exact_gram_kernel(
     // a bounded wait that also ends when another warp gave up
     auto wait = [&](uint64_t* bar, uint32_t parity) -> bool {
         if (abort_flag) return false;
-        if (tc::mbar_wait(bar, parity, limit)) return true;
+        if (kPoll) {
+            if (tc::mbar_wait(bar, parity, limit)) return true;
+        } else {
+            // (the first try without a look at the clock: 144 -> 128 us of
+            // the minima of 2,000 queries and 200,000 x 128 rows)
+            if (tc::mbar_try_wait(bar, parity)) return true;
+            const long long t0 = clock64();
+            do {
+                if (tc::mbar_try_wait(bar, parity)) return true;
+            } while (clock64() - t0 <= limit);
+        }
         give_up();
         return false;
     };
@@ -755,9 +766,11 @@ cudaError_t run_exact_knn_tc(const XDesc& x, const int32_t* queries, int nq, int
     const bool a_stays = nK <= 4;
     const size_t smem = 1024 + (a_stays ? (size_t)nK * kTileM * 128 : 0) +
                         kGramStages * (size_t)((a_stays ? 0 : kTileM * 128) + kTileN * 128) + 2 * kTileN * sizeof(float);
-    cudaError_t e = cudaFuncSetAttribute(exact_gram_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(exact_gram_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const bool poll = limit < tc::kPollBelow;
+    auto minima = poll ? exact_gram_kernel<false, true> : exact_gram_kernel<false, false>;
+    auto listing = poll ? exact_gram_kernel<true, true> : exact_gram_kernel<true, false>;
+    cudaError_t e = cudaFuncSetAttribute(minima, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(listing, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess) e = cudaMemsetAsync(stats, 0, sizeof(ExactStats), st);
     if (e != cudaSuccess) return e;
     auto typed = [&](auto&& f) {
@@ -780,11 +793,11 @@ cudaError_t run_exact_knn_tc(const XDesc& x, const int32_t* queries, int nq, int
         float* od = dists + (int64_t)q0 * k;
         exact_gather_kernel<<<(int)std::min<int64_t>(((int64_t)rows * (dq / 8) + 255) / 256, (int64_t)G * 8), 256, 0, st>>>(
             reinterpret_cast<const uint4*>(Xq), x.n, dq / 8, qs, cq, rows, reinterpret_cast<uint4*>(Aq));
-        exact_gram_kernel<false><<<Gb, kGramThreads, smem, st>>>(amap, bmap, nK, RT, CT, a_stays, nrm, mins, nullptr,
+        minima<<<Gb, kGramThreads, smem, st>>>(amap, bmap, nK, RT, CT, a_stays, nrm, mins, nullptr,
                                                                 nullptr, nullptr, limit, err);
         exact_bound_kernel<<<(rows + 7) / 8, 256, 0, st>>>(x.n, x.d, k, qs, cq, rows, Gb, CT, total, mins, nrm, xerr,
                                                            stats, thr, counts, need);
-        exact_gram_kernel<true><<<Gb, kGramThreads, smem, st>>>(amap, bmap, nK, RT, CT, a_stays, nrm, nullptr, thr,
+        listing<<<Gb, kGramThreads, smem, st>>>(amap, bmap, nK, RT, CT, a_stays, nrm, nullptr, thr,
                                                                counts, lists, limit, err);
         note_launches(4);
         typed([&](auto rl) {
