@@ -13,7 +13,9 @@
 //
 // The filtered form (run_exact_knn_tc) scores the pairs on the tensor cores
 // and computes the canonical distance only of those that can be listed:
-//   1. x^ = bfloat16(x) of every row, |x^|^2 and the distance |x - x^|;
+//   1. x^ = bfloat16(x) of every row, |x^|^2 and the distance |x - x^|; rows
+//      far above the others by either are taken out and listed for every
+//      query;
 //   2. exact_gram_kernel (minima): D^ = |q^|^2 + |x^|^2 - 2 q^.x^ of every
 //      pair (tcgen05, FP32 accumulation), reduced to minima over 64 groups of
 //      rows per query and CTA;
@@ -28,8 +30,13 @@
 //      (a few tens on descriptor data);
 //   5. exact_rescore_kernel: canonical distances of the listed rows, the k
 //      best by (distance, id).
-// Queries whose list overflows, and all of them when a row is not finite or a
-// bounded wait gave up, are answered by exact_knn_kernel.
+// Queries whose list overflows or whose own row is a far one, and all of them
+// when more rows are not finite than can be taken out or a bounded wait gave
+// up, are answered by exact_knn_kernel.  One row 300 times longer than the
+// rest (2,000 queries of 200,000 x 128): 52.7 -> 0.6 ms.  What the bounds
+// cannot help (more than 1,024 rows nearly as near as the k-th, rows far from
+// the origin for their spread) costs the passes beside the direct kernel: 12 %
+// at 2,048 rows and 10 queries, 3 % at 16,384 and 1,000, 1 % at 200,000.
 // 10,000 queries of 1,000,000 x 128 rows, k = 20: 788 ms with exact_knn_kernel
 // alone (seven shuffles per pair and 128 entries), 7.6 ms filtered.
 #include <cuda.h>
@@ -204,37 +211,46 @@ constexpr int kRescoreWarps = 4;
 constexpr long long kExactWait = 2000000000LL;  // ~1 s at GB300 clocks: the default limit of the
                                                 // waits, and the limit of the drains
 
-// Largest |x - x^| and |x^|^2 over the rows (as order-preserving words of
-// non-negative floats) and whether a row is not finite.
+// The bounds use the largest |x - x^| and |x^|^2 over the rows, so rows far
+// above the others (and rows that are not finite) are taken out: at most
+// kFarRows by either measure.  They are listed for every query instead.
+constexpr int kFarRows = 64;
+constexpr int kUnusable = 255;  // histogram bin of rows that no bound holds for
+
+// Over the rows: histograms of the exponents of |x^|^2 and |x - x^|; the rows
+// taken out and the largest values of the others (as order-preserving words
+// of non-negative floats); bad: more unusable rows than can be taken out.
 struct ExactStats {
     uint32_t max_err;
     uint32_t max_nrm;
     uint32_t bad;
-    uint32_t pad;
+    uint32_t nfar;
+    int32_t far[2 * kFarRows];
+    uint32_t nrm_hist[256];
+    uint32_t err_hist[256];
 };
 }  // namespace
 
-// One warp per row: bfloat16 copy (rows of dq entries, zeros past d), squared
-// norm of the copy, distance to it.  Norms of the padding rows are +inf.
-template <int kDT>
+// kLanes lanes a row: bfloat16 copy (rows of dq entries, zeros past d), squared
+// norm of the copy, distance to it.  Norms of unusable rows and of the padding
+// rows are +inf: neither pass finds them.
+// kLanes: lanes a row, 16 for rows of one K slice (10 queries of 500,000 x 64
+// bytes: 266 -> 234 us).
+template <int kDT, int kLanes>
 __global__ void __launch_bounds__(256) exact_quant_kernel(RowLoader<kDT> L, int64_t n, int64_t n_pad, int dq,
                                                           __nv_bfloat16* __restrict__ Xq, float* __restrict__ nrm,
-                                                          float* __restrict__ err, ExactStats* __restrict__ stats)
+                                                          float* __restrict__ err)
 {
-    const int lane = threadIdx.x & 31;
-    const int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    float me = 0.f, mn = 0.f;
-    bool bad = false;
+    const int lane = threadIdx.x & (kLanes - 1);
+    const int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / kLanes;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) / kLanes;
+    // (n_pad and nw are even: a warp's groups go round together)
     for (int64_t r = gw; r < n_pad; r += nw) {
-        if (r >= n) {
-            if (lane == 0) nrm[r] = __int_as_float(0x7f800000);
-            continue;
-        }
+        const int64_t row = r < n ? r : n - 1;  // (padding: the last row once more)
         float s = 0.f, e = 0.f;
-        __nv_bfloat16* o = Xq + r * dq;
-        for (int j = 4 * lane; j < dq; j += 128) {
-            const float4 v = j < L.d ? L.load4(r, j) : make_float4(0.f, 0.f, 0.f, 0.f);
+        __nv_bfloat16* o = Xq + row * dq;
+        for (int j = 4 * lane; j < dq; j += 4 * kLanes) {
+            float4 v = j < L.d ? L.load4(row, j) : make_float4(0.f, 0.f, 0.f, 0.f);
             const __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
             const float2 fa = __bfloat1622float2(a), fb = __bfloat1622float2(b);
             s = fmaf(fa.x, fa.x, s); s = fmaf(fa.y, fa.y, s);
@@ -250,34 +266,81 @@ __global__ void __launch_bounds__(256) exact_quant_kernel(RowLoader<kDT> L, int6
             *reinterpret_cast<uint2*>(o + j) = u;
         }
 #pragma unroll
-        for (int q = 16; q >= 1; q >>= 1) {
+        for (int q = kLanes / 2; q >= 1; q >>= 1) {
             s += __shfl_xor_sync(KNNG_FULL_MASK, s, q);
             e += __shfl_xor_sync(KNNG_FULL_MASK, e, q);
+        }
+        if (r >= n) {
+            if (lane == 0) nrm[r] = __int_as_float(0x7f800000);
+            continue;
         }
         // (rounded up: the sum's relative error is below (d / 32 + 8) 2^-24,
         // and squares that underflow lose d 2^-149 <= 2^-138 in all)
         e = sqrtf(e) * 1.0001f + 0x1p-69f;
         if (lane == 0) {
-            nrm[r] = s;
+            // 1e30 also keeps the bounds' squares finite
+            nrm[r] = s <= 1e30f && e <= 1e30f ? s : __int_as_float(0x7f800000);
             err[r] = e;
         }
-        // 1e30 also keeps the bounds' squares finite
-        bad |= !(s <= 1e30f) || !(e <= 1e30f);
-        me = fmaxf(me, e);
-        mn = fmaxf(mn, s);
-    }
-    if (lane == 0) {
-        atomicMax(&stats->max_err, __float_as_uint(me));
-        atomicMax(&stats->max_nrm, __float_as_uint(mn));
-        if (bad) atomicOr(&stats->bad, 1u);
     }
 }
 
-// The batch's query rows, packed (rows of dq entries; zeros past nq and for
-// ids out of range).
-__global__ void __launch_bounds__(256) exact_gather_kernel(const uint4* __restrict__ Xq, int64_t n, int row16,
-                                                           const int32_t* __restrict__ queries, int nq, int rows,
-                                                           uint4* __restrict__ Aq)
+// Histograms of the exponents of the norms and errors.  (A kernel of its own:
+// counted by the one above, whose rows are a chain of loads and shuffles at
+// 32 registers, 1M x 100 took 179 to 222 us there instead of 160.)
+__global__ void __launch_bounds__(256) exact_hist_kernel(int64_t n, const float* __restrict__ nrm,
+                                                         const float* __restrict__ err, ExactStats* __restrict__ stats)
+{
+    __shared__ uint32_t hist[512];
+    for (int i = threadIdx.x; i < 512; i += 256) hist[i] = 0u;
+    __syncthreads();
+    for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < n; r += (int64_t)gridDim.x * blockDim.x) {
+        const float s = nrm[r], e = err[r];
+        atomicAdd(&hist[s <= 1e30f ? __float_as_uint(s) >> 23 : kUnusable], 1u);
+        if (s <= 1e30f) atomicAdd(&hist[256 + (__float_as_uint(e) >> 23)], 1u);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < 512; i += 256)
+        if (hist[i]) atomicAdd(i < 256 ? &stats->nrm_hist[i] : &stats->err_hist[i - 256], hist[i]);
+}
+
+// One warp: the exponent above which a histogram's rows are taken out.  Those
+// above the smallest exponent with at most kFarRows rows past it, if that
+// leaves the usable ones at least 2^(gap - 1) times smaller; else unusable
+// rows only.
+__device__ __forceinline__ int far_cut(const uint32_t* __restrict__ hist, int gap)
+{
+    const int lane = threadIdx.x & 31;
+    uint32_t c[8], sum = 0;
+    int top = -1;
+#pragma unroll
+    for (int b = 0; b < 8; ++b) {
+        c[b] = hist[8 * lane + b];
+        sum += c[b];
+        if (c[b] && 8 * lane + b < kUnusable) top = 8 * lane + b;
+    }
+    top = __reduce_max_sync(KNNG_FULL_MASK, top);
+    uint32_t past = sum;  // rows of this lane's bins and above
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t v = __shfl_down_sync(KNNG_FULL_MASK, past, o);
+        if (lane + o < 32) past += v;
+    }
+    past -= sum;
+    int least = 256;
+#pragma unroll
+    for (int b = 7; b >= 0; --b) {
+        if (past <= kFarRows) least = 8 * lane + b;
+        past += c[b];
+    }
+    least = __reduce_min_sync(KNNG_FULL_MASK, least);
+    return top - least >= gap ? least : kUnusable - 1;
+}
+
+// The batch's query rows, packed (rows of row16 16-byte words; zeros past nq
+// and for ids out of range).
+__device__ __forceinline__ void gather_queries(const uint4* __restrict__ Xq, int64_t n, int row16,
+                                               const int32_t* __restrict__ queries, int nq, int rows,
+                                               uint4* __restrict__ Aq)
 {
     const int64_t total = (int64_t)rows * row16;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
@@ -285,6 +348,61 @@ __global__ void __launch_bounds__(256) exact_gather_kernel(const uint4* __restri
         const int r = (int)(e / row16), c = (int)(e - (int64_t)r * row16);
         const int32_t q = r < nq ? queries[r] : -1;
         Aq[e] = q >= 0 && q < n ? Xq[(int64_t)q * row16 + c] : make_uint4(0u, 0u, 0u, 0u);
+    }
+}
+__global__ void __launch_bounds__(256) exact_gather_kernel(const uint4* __restrict__ Xq, int64_t n, int row16,
+                                                           const int32_t* __restrict__ queries, int nq, int rows,
+                                                           uint4* __restrict__ Aq)
+{
+    gather_queries(Xq, n, row16, queries, nq, rows, Aq);
+}
+
+// Takes the far rows out (norm +inf) and finds the largest norm and error of
+// the others.  A factor of 8 in the squared norm or of 2 in the error pays for
+// kFarRows more rescored rows a query.  Gathers the first batch's queries as
+// well (a launch less).
+__global__ void __launch_bounds__(256) exact_far_kernel(int64_t n, float* __restrict__ nrm,
+                                                        const float* __restrict__ err, ExactStats* __restrict__ stats,
+                                                        const uint4* __restrict__ Xq, int row16,
+                                                        const int32_t* __restrict__ queries, int nq, int rows,
+                                                        uint4* __restrict__ Aq)
+{
+    gather_queries(Xq, n, row16, queries, nq, rows, Aq);
+    __shared__ int cut[2];
+    __shared__ uint32_t most[2][8];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (w < 2) {
+        const int c = w == 0 ? far_cut(stats->nrm_hist, 4) : far_cut(stats->err_hist, 2);
+        if (lane == 0) cut[w] = c;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) stats->bad = stats->nrm_hist[kUnusable] > kFarRows ? 1u : 0u;
+    __syncthreads();
+    float me = 0.f, mn = 0.f;
+    for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < n; r += (int64_t)gridDim.x * blockDim.x) {
+        const float s = nrm[r], e = err[r];
+        const bool usable = s <= 1e30f;
+        if (!usable || (int)(__float_as_uint(s) >> 23) > cut[0] || (int)(__float_as_uint(e) >> 23) > cut[1]) {
+            const uint32_t at = atomicAdd(&stats->nfar, 1u);
+            if (at < 2 * kFarRows) stats->far[at] = (int32_t)r;
+            nrm[r] = __int_as_float(0x7f800000);
+        } else {
+            me = fmaxf(me, e);
+            mn = fmaxf(mn, s);
+        }
+    }
+    for (int o = 16; o >= 1; o >>= 1) {
+        me = fmaxf(me, __shfl_xor_sync(KNNG_FULL_MASK, me, o));
+        mn = fmaxf(mn, __shfl_xor_sync(KNNG_FULL_MASK, mn, o));
+    }
+    if (lane == 0) {
+        most[0][w] = __float_as_uint(me);
+        most[1][w] = __float_as_uint(mn);
+    }
+    __syncthreads();
+    if (threadIdx.x < 2) {
+        uint32_t m = 0u;
+        for (int i = 0; i < 8; ++i) m = max(m, most[threadIdx.x][i]);
+        atomicMax(threadIdx.x == 0 ? &stats->max_err : &stats->max_nrm, m);
     }
 }
 
@@ -310,7 +428,7 @@ __host__ __device__ __forceinline__ int64_t tile_begin(int64_t total, int G, int
 //   holds back cost the products, not an atomic per pair.  2,000 queries of
 //   200,000 x 128 equal rows, which the direct kernel answers in 52.2 ms: 56.7
 //   in all with an atomic per pair, 52.6 so.
-// A set with a row that is not usable takes the direct kernel: both passes
+// A set with too many unusable rows takes the direct kernel: both passes
 // return at once (52.7 -> 52.5 ms).
 // kPoll: the waits poll without suspending (limits too short for try_wait).
 template <bool kList, bool kPoll>
@@ -578,7 +696,7 @@ __global__ void __launch_bounds__(kGramThreads, 1) exact_gram_kernel(
 }
 
 // One warp per query: the bound of step 3 as a limit of |x^|^2 - 2 q^.x^ (in
-// thr; -inf: nothing is listed), the list count reset, and the mark of
+// thr; -inf: nothing is listed), the list with the far rows, and the mark of
 // queries left to exact_knn_kernel.
 __global__ void __launch_bounds__(256) exact_bound_kernel(int64_t n, int d, int k, const int32_t* __restrict__ queries,
                                                           int nq, int rows, int G, int CT, int64_t total,
@@ -586,7 +704,7 @@ __global__ void __launch_bounds__(256) exact_bound_kernel(int64_t n, int d, int 
                                                           const float* __restrict__ nrm, const float* __restrict__ err,
                                                           const ExactStats* __restrict__ stats,
                                                           float* __restrict__ thr, int* __restrict__ counts,
-                                                          uint8_t* __restrict__ need)
+                                                          int32_t* __restrict__ lists, uint8_t* __restrict__ need)
 {
     __shared__ uint32_t hist_all[8][256];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -597,7 +715,7 @@ __global__ void __launch_bounds__(256) exact_bound_kernel(int64_t n, int d, int 
     const bool valid = q >= 0 && q < n;
     float lim = -kInf;
     bool left = false;
-    if (valid && stats->bad) left = true;
+    if (valid && (stats->bad || !(nrm[q] <= 1e30f))) left = true;  // (its own row is a far one)
     if (valid && !left) {
         // the CTAs with tiles of this query's row tile
         const int rt = qi / kTileM, lr = qi % kTileM;
@@ -645,9 +763,12 @@ __global__ void __launch_bounds__(256) exact_bound_kernel(int64_t n, int d, int 
             left = true;
         }
     }
+    // the far rows are listed at once
+    const int nfar = valid && !left ? (int)stats->nfar : 0;
+    for (int i = lane; i < nfar; i += 32) lists[(int64_t)qi * kListMax + i] = stats->far[i];
     if (lane == 0) {
         thr[qi] = lim;
-        counts[qi] = 0;
+        counts[qi] = nfar;
         if (qi < nq) need[qi] = left ? 1 : 0;
     }
 }
@@ -739,6 +860,9 @@ static bool exact_rows_map(CUtensorMap* map, void* base, int dq, int64_t rows, i
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+template <int kDT>
+std::integral_constant<int, kDT> dtype_of(const RowLoader<kDT>&);
+
 // The filtered form from 2,048 rows on: exact_knn_kernel streams all rows per
 // block, 0.51 ms at 2,048 x 128 for 10 or 1,000 queries and 3.8 ms at 16,384,
 // the filtered form 0.09 / 0.12 ms and 0.15 / 0.19 ms; smaller sets keep the
@@ -793,10 +917,15 @@ cudaError_t run_exact_knn_tc(const XDesc& x, const int32_t* queries, int nq, int
         else f(RowLoader<kDtF32>{x.X, x.ld, x.d, x.vec});
     };
     typed([&](auto rl) {
+        constexpr int kDT = decltype(dtype_of(rl))::value;
         const int grid = (int)std::min<int64_t>((n_pad + 7) / 8, (int64_t)G * 8);
-        exact_quant_kernel<<<grid, 256, 0, st>>>(rl, x.n, n_pad, dq, Xq, nrm, xerr, stats);
-        note_launches(1);
+        auto quant = dq == 64 ? exact_quant_kernel<kDT, 16> : exact_quant_kernel<kDT, 32>;
+        quant<<<grid, 256, 0, st>>>(rl, x.n, n_pad, dq, Xq, nrm, xerr);
     });
+    exact_hist_kernel<<<(int)std::min<int64_t>((x.n + 255) / 256, (int64_t)G * 2), 256, 0, st>>>(x.n, nrm, xerr, stats);
+    exact_far_kernel<<<G * 2, 256, 0, st>>>(x.n, nrm, xerr, stats, reinterpret_cast<const uint4*>(Xq), dq / 8, queries,
+                                           bq, brows, reinterpret_cast<uint4*>(Aq));
+    note_launches(3);
     for (int q0 = 0; q0 < nq; q0 += kBatchQ) {
         const int cq = std::min(nq - q0, kBatchQ);
         const int RT = (cq + kTileM - 1) / kTileM, rows = RT * kTileM;
@@ -805,15 +934,19 @@ cudaError_t run_exact_knn_tc(const XDesc& x, const int32_t* queries, int nq, int
         const int32_t* qs = queries + q0;
         int32_t* oi = ids + (int64_t)q0 * k;
         float* od = dists + (int64_t)q0 * k;
-        exact_gather_kernel<<<(int)std::min<int64_t>(((int64_t)rows * (dq / 8) + 255) / 256, (int64_t)G * 8), 256, 0, st>>>(
-            reinterpret_cast<const uint4*>(Xq), x.n, dq / 8, qs, cq, rows, reinterpret_cast<uint4*>(Aq));
+        if (q0 > 0) {
+            const int grid = (int)std::min<int64_t>(((int64_t)rows * (dq / 8) + 255) / 256, (int64_t)G * 8);
+            exact_gather_kernel<<<grid, 256, 0, st>>>(reinterpret_cast<const uint4*>(Xq), x.n, dq / 8, qs, cq, rows,
+                                                      reinterpret_cast<uint4*>(Aq));
+            note_launches(1);
+        }
         minima<<<Gb, kGramThreads, smem, st>>>(amap, bmap, nK, RT, CT, a_stays, nrm, stats, mins, nullptr,
                                                                 nullptr, nullptr, limit, err);
         exact_bound_kernel<<<(rows + 7) / 8, 256, 0, st>>>(x.n, x.d, k, qs, cq, rows, Gb, CT, total, mins, nrm, xerr,
-                                                           stats, thr, counts, need);
+                                                           stats, thr, counts, lists, need);
         listing<<<Gb, kGramThreads, smem, st>>>(amap, bmap, nK, RT, CT, a_stays, nrm, stats, nullptr, thr,
                                                                counts, lists, limit, err);
-        note_launches(4);
+        note_launches(3);
         typed([&](auto rl) {
             exact_rescore_kernel<<<(cq + kRescoreWarps - 1) / kRescoreWarps, kRescoreWarps * 32, 0, st>>>(
                 rl, x.n, qs, cq, k, counts, lists, need, err, oi, od);

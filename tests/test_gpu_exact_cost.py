@@ -46,7 +46,19 @@ def test_handed_back_sets_cost_the_direct_form(kind):
     if kind == "equal":
         X[:] = X[0].clone()
     else:
-        X[::2, 1] = float("nan")
+        X[::2, 1] = float("nan")  # (far more rows than can be taken out)
     q = torch.arange(nq, dtype=torch.int32, device="cuda") * (n // nq)
     call, direct = call_and_direct(X, q, 10)
     assert call < 1.05 * direct
+
+
+@pytest.mark.parametrize("kind", ["one long row", "one infinite row"])
+def test_one_odd_row_leaves_the_filter_to_the_others(kind):
+    # the bound of every query took its margins from the largest row: all
+    # queries went to the direct form
+    n, nq = 60000, 2000
+    X = normal_rows(n, 64, 2)
+    X[n // 2] = X[n // 2] * 300.0 if kind == "one long row" else float("inf")
+    q = torch.arange(nq, dtype=torch.int32, device="cuda") * (n // nq) + 1
+    call, direct = call_and_direct(X, q, 10)
+    assert call < 0.5 * direct

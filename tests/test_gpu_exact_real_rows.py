@@ -68,3 +68,23 @@ def test_rows_of_very_small_magnitude(d, scale):
     # bound what they lose
     X = (np.random.default_rng(d).standard_normal((2048, d)) * scale).astype(np.float32)
     check(X, np.arange(0, 2048, 7), 10)
+
+
+@pytest.mark.parametrize("count", [1, 2, 63, 64, 65, 300])
+@pytest.mark.parametrize("kind", ["long", "not finite", "inexact", "long and not finite"])
+def test_rows_far_above_the_others(kind, count):
+    # up to 64 such rows are taken out of the bounds and listed for every
+    # query, more loosen the bounds (long rows, rows bfloat16 does not hold)
+    # or send all queries to the direct form (rows that are not finite).  The
+    # far rows are near one another, and some are queries.
+    rng = np.random.default_rng(count)
+    n, d = 4000, 24
+    X = rng.integers(-100, 101, size=(n, d)).astype(np.float32)
+    far = rng.choice(n, size=count, replace=False)
+    if kind != "not finite":
+        X[far] = (37.3 + rng.standard_normal((count, d))) * (1.0 if kind == "inexact" else 5000.0)
+    if kind in ("not finite", "long and not finite"):
+        for i in far[::2] if kind == "long and not finite" else far:
+            X[i, rng.integers(d)] = (np.inf, -np.inf, np.nan, 3e38)[rng.integers(4)]
+    q = np.unique(np.r_[rng.choice(n, size=150), far[:20]])
+    check(X, q, 15)
