@@ -51,6 +51,10 @@ struct BatchCache {
     cudaStream_t cap = nullptr;
     cudaEvent_t ev_in = nullptr, ev_out = nullptr;
     int kernels = 0;  // kernel nodes of the graph
+    // the workspace the graph was recorded in: another call may have grown
+    // (and so moved) the handle's since
+    const char* ws = nullptr;
+    size_t ws_need = 0;
 };
 
 struct knng_handle {
@@ -978,7 +982,7 @@ int knng_build_batched(knng_handle* h, int32_t nsets, const knng_dataset* sets, 
             return fail(h, KNNG_ERR_CUDA, "batch stream / events");
         }
     }
-    if (!B.exec || sig != B.sig) {
+    if (!B.exec || sig != B.sig || B.ws != h->ws || B.ws_need > h->ws_size) {
         // ---- record the batch: groups of equal (dtype, d) form one forest
         if (B.exec) { cudaGraphExecDestroy(B.exec); B.exec = nullptr; }
         if (B.graph) { cudaGraphDestroy(B.graph); B.graph = nullptr; }
@@ -1103,6 +1107,8 @@ int knng_build_batched(knng_handle* h, int32_t nsets, const knng_dataset* sets, 
         }
         B.graph = graph;
         B.sig = sig;
+        B.ws = h->ws;
+        B.ws_need = need;
     }
     // ---- one graph launch, ordered after and before the caller's stream
     cudaError_t e = cudaEventRecord(B.ev_in, st);
