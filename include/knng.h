@@ -29,7 +29,8 @@
  *    and nothing throws across the ABI.  knng_last_error() describes the last
  *    failure of a handle.
  *  - A handle owns a device workspace, grown on demand with the stream-ordered
- *    allocator; calls on one handle must not run concurrently from several
+ *    allocator (without memory for it, the stages take forms that need less
+ *    and are slower; KNNG_ERR_OOM when these do not fit either); calls on one handle must not run concurrently from several
  *    host threads.
  */
 #ifndef KNNG_H
@@ -414,11 +415,13 @@ int knng_normalize_rows(knng_handle* h, const void* X, int32_t dtype, int64_t n,
  * accuracy measure of Sec. 4).  queries: device int32 [nq] point ids;
  * ids, dists: device [nq][k], ordered by (distance, id).
  * From 2,048 points on, pairs that cannot be listed are ruled out by a
- * tensor-core pass with a proven bound first (same lists); its scratch -- a
- * bfloat16 copy of X and up to 64 MB -- is kept by the handle, and the calls
- * of one handle on several streams are ordered by an event.  A call on a
- * stream that is being captured, or without memory for the scratch, takes
- * the direct form. */
+ * tensor-core pass with a proven bound first (same lists).  Its scratch is a
+ * bfloat16 copy of X (rows padded to a multiple of 64 entries), 8 bytes a row
+ * and up to 140 MB for a batch of queries, an eighth more to grow in.  The
+ * handle keeps it, and gives it back when another allocation of the handle
+ * fails; the calls of one handle on several streams are ordered by an event.
+ * A call on a stream that is being captured, or without memory for the
+ * scratch, takes the direct form. */
 int knng_exact_knn(knng_handle* h, const void* X, int32_t dtype, int64_t n, int32_t d, int64_t ld,
                    const int32_t* queries, int64_t nq, int32_t k, int32_t* ids, float* dists,
                    void* stream);

@@ -120,7 +120,34 @@ struct DeviceGuard {
     }
 };
 
-// Grows the workspace to at least `bytes` (stream-ordered free/alloc).
+bool capturing(cudaStream_t st)
+{
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cs) == cudaSuccess) return cs != cudaStreamCaptureStatusNone;
+    cudaGetLastError();
+    return true;
+}
+
+// Stream-ordered allocation for the handle.  Short of memory, the scratch
+// that knng_exact_knn keeps is given back first.
+cudaError_t handle_alloc(knng_handle* h, void** p, size_t bytes, cudaStream_t st)
+{
+    cudaError_t e = cudaMallocAsync(p, bytes, st);
+    if (e == cudaSuccess || capturing(st)) return e;
+    cudaGetLastError();
+    if (h->exact_ws && cudaStreamWaitEvent(st, h->exact_done, 0) == cudaSuccess) {
+        cudaFreeAsync(h->exact_ws, st);
+        h->exact_ws = nullptr;
+        h->exact_ws_size = 0;
+    }
+    cudaStreamSynchronize(st);  // what was freed on the stream goes back to the device
+    e = cudaMallocAsync(p, bytes, st);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
+}
+
+// Grows the workspace to at least `bytes` (stream-ordered free/alloc): with
+// room to grow, or without when there is no memory for it.
 int ensure_ws(knng_handle* h, size_t bytes, cudaStream_t st)
 {
     if (bytes <= h->ws_size) return KNNG_OK;
@@ -131,13 +158,38 @@ int ensure_ws(knng_handle* h, size_t bytes, cudaStream_t st)
     }
     size_t want = bytes + (bytes >> 3) + (1 << 20);
     void* p = nullptr;
-    cudaError_t e = cudaMallocAsync(&p, want, st);
+    cudaError_t e = handle_alloc(h, &p, want, st);
+    if (e != cudaSuccess) {
+        want = bytes;
+        e = handle_alloc(h, &p, want, st);
+    }
     if (e != cudaSuccess) {
         cudaGetLastError();
         return fail(h, KNNG_ERR_OOM, "workspace of %zu bytes: %s", want, cudaGetErrorString(e));
     }
     h->ws = static_cast<char*>(p);
     h->ws_size = want;
+    return KNNG_OK;
+}
+
+// Makes room for a call's workspace and starts a at it.  measure(m) carves the
+// workspace from a measuring arena; without memory for it -- or, while st is
+// being captured, without room for it -- the stages' forms that need less
+// scratch are measured and taken (Arena::lean).
+template <class Measure>
+int take_ws(knng_handle* h, cudaStream_t st, Arena& a, Measure measure)
+{
+    Arena full, small;
+    small.lean = true;
+    int r;
+    if ((r = measure(full)) || (r = measure(small))) return r;
+    // (a stage that needs no scratch still runs with a base, not as a measurement)
+    const size_t need = std::max<size_t>(full.off, 1), least = std::max<size_t>(small.off, 1);
+    a = Arena{};
+    if (need > h->ws_size && least < need)
+        a.lean = capturing(st) ? least <= h->ws_size : ensure_ws(h, need, st) != KNNG_OK;
+    if ((r = ensure_ws(h, a.lean ? least : need, st))) return r;
+    a.base = h->ws;
     return KNNG_OK;
 }
 
@@ -192,11 +244,7 @@ int ensure_plan(knng_handle* h, int64_t n, int g, cudaStream_t st)
 // that needs none.
 bool exact_scratch(knng_handle* h, const XDesc& x, int nq, int k, cudaStream_t st)
 {
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
-        cudaGetLastError();
-        return false;
-    }
+    if (capturing(st)) return false;
     if (!h->exact_done && cudaEventCreateWithFlags(&h->exact_done, cudaEventDisableTiming) != cudaSuccess) {
         cudaGetLastError();
         h->exact_done = nullptr;
@@ -599,11 +647,12 @@ int knng_partition(knng_handle* h, const void* X, int32_t dtype, int64_t n, int3
     DeviceGuard dg(h->device);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if ((r = ensure_plan(h, n, g, st))) return r;
-    Arena m;
-    run_partition(x, h->plan, h->dplan, T, seed, perm, m, st);
-    if ((r = ensure_ws(h, m.off, st))) return r;
     Arena a;
-    a.base = h->ws;
+    if ((r = take_ws(h, st, a, [&](Arena& m) {
+            run_partition(x, h->plan, h->dplan, T, seed, nullptr, m, st);
+            return KNNG_OK;
+        })))
+        return r;
     cudaError_t e = run_partition(x, h->plan, h->dplan, T, seed, perm, a, st, nullptr, 0, nullptr, h->dev_err);
     if (e != cudaSuccess) return cuda_fail(h, e, "partition");
     return KNNG_OK;
@@ -634,11 +683,12 @@ int knng_partition_pca(knng_handle* h, const void* X, int32_t dtype, int64_t n, 
     pca.on = true;
     pca.out = dirs_out;
     pca.stride = ((((int64_t)1) << h->plan.levels.size()) - 1) * d;
-    Arena m;
-    run_partition(x, h->plan, h->dplan, T, seed, nullptr, m, st, nullptr, 0, &pca);
-    if ((r = ensure_ws(h, m.off, st))) return r;
     Arena a;
-    a.base = h->ws;
+    if ((r = take_ws(h, st, a, [&](Arena& m) {
+            run_partition(x, h->plan, h->dplan, T, seed, nullptr, m, st, nullptr, 0, &pca);
+            return KNNG_OK;
+        })))
+        return r;
     const cudaError_t e = run_partition(x, h->plan, h->dplan, T, seed, perm, a, st, nullptr, 0, &pca, h->dev_err);
     if (e != cudaSuccess) return cuda_fail(h, e, "partition");
     return KNNG_OK;
@@ -658,12 +708,11 @@ int knng_leaf_knn(knng_handle* h, const void* X, int32_t dtype, int64_t n, int32
     DeviceGuard dg(h->device);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if ((r = ensure_plan(h, n, g, st))) return r;
-    Arena m;
-    if ((r = leaf_stage(h, h->plan, h->dplan, x, T, perm, k, precision, rescore_mult, ids, dists, m, st))) return r;
-    // (a stage that needs no scratch still runs with a base, not as a measurement)
-    if ((r = ensure_ws(h, std::max<size_t>(m.off, 1), st))) return r;
     Arena a;
-    a.base = h->ws;
+    if ((r = take_ws(h, st, a, [&](Arena& m) {
+            return leaf_stage(h, h->plan, h->dplan, x, T, perm, k, precision, rescore_mult, ids, dists, m, st);
+        })))
+        return r;
     return leaf_stage(h, h->plan, h->dplan, x, T, perm, k, precision, rescore_mult, ids, dists, a, st);
 }
 
@@ -831,11 +880,11 @@ int knng_build(knng_handle* h, const void* X, int32_t dtype, int64_t n, int32_t 
     DeviceGuard dg(h->device);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if ((r = ensure_plan(h, n, p->leaf_size, st))) return r;
-    Arena m;
-    if ((r = build_pipeline(h, h->plan, h->dplan, x, *p, ids, dists, m, st, true, nullptr, true))) return r;
-    if ((r = ensure_ws(h, m.off, st))) return r;
     Arena a;
-    a.base = h->ws;
+    if ((r = take_ws(h, st, a, [&](Arena& m) {
+            return build_pipeline(h, h->plan, h->dplan, x, *p, ids, dists, m, st, true, nullptr, true);
+        })))
+        return r;
     return build_pipeline(h, h->plan, h->dplan, x, *p, ids, dists, a, st, true, nullptr, true);
 }
 
@@ -1052,18 +1101,25 @@ int knng_build_batched(knng_handle* h, int32_t nsets, const knng_dataset* sets, 
             g.dev_sets = reinterpret_cast<const BatchSet*>(B.tables + offs[4 * gi + 3]);
         }
         // workspace: the largest group (groups run one after another)
-        size_t need = 0;
-        for (BatchGroup& g : B.groups) {
-            Arena m;
-            const size_t es = dtype_size(g.dtype);
-            m.take<char>((size_t)g.n * g.ld * es);
-            m.take<int32_t>((size_t)g.n * p->k);
-            m.take<float>((size_t)g.n * p->k);
-            XDesc x{nullptr, g.dtype, g.n, g.d, g.ld, true};
-            if ((r = build_pipeline(h, g.plan, g.dp, x, *p, nullptr, nullptr, m, st, false))) return r;
-            need = std::max(need, m.off);
-        }
-        if ((r = ensure_ws(h, need, st))) return r;
+        Arena ws;
+        if ((r = take_ws(h, st, ws, [&](Arena& all) {
+                size_t need = 0;
+                for (BatchGroup& g : B.groups) {
+                    Arena m;
+                    m.lean = all.lean;
+                    const size_t es = dtype_size(g.dtype);
+                    m.take<char>((size_t)g.n * g.ld * es);
+                    m.take<int32_t>((size_t)g.n * p->k);
+                    m.take<float>((size_t)g.n * p->k);
+                    XDesc x{nullptr, g.dtype, g.n, g.d, g.ld, true};
+                    const int e = build_pipeline(h, g.plan, g.dp, x, *p, nullptr, nullptr, m, st, false);
+                    if (e) return e;
+                    need = std::max(need, m.off);
+                }
+                all.off = need;
+                return KNNG_OK;
+            })))
+            return r;
         if (cudaStreamSynchronize(st) != cudaSuccess) return cuda_fail(h, cudaGetLastError(), "batch setup");
         // record every group's pipeline into one graph
         if (cudaStreamBeginCapture(B.cap, cudaStreamCaptureModeThreadLocal) != cudaSuccess)
@@ -1071,8 +1127,7 @@ int knng_build_batched(knng_handle* h, int32_t nsets, const knng_dataset* sets, 
         int rr = KNNG_OK;
         const unsigned long long c0 = launch_count();
         for (BatchGroup& g : B.groups) {
-            Arena a;
-            a.base = h->ws;
+            Arena a = ws;
             const size_t es = dtype_size(g.dtype);
             char* xc = a.take<char>((size_t)g.n * g.ld * es);
             int32_t* gi = a.take<int32_t>((size_t)g.n * p->k);
@@ -1108,7 +1163,7 @@ int knng_build_batched(knng_handle* h, int32_t nsets, const knng_dataset* sets, 
         B.graph = graph;
         B.sig = sig;
         B.ws = h->ws;
-        B.ws_need = need;
+        B.ws_need = h->ws_size;
     }
     // ---- one graph launch, ordered after and before the caller's stream
     cudaError_t e = cudaEventRecord(B.ev_in, st);
@@ -1137,18 +1192,21 @@ int knng_autotune(knng_handle* h, const void* X, int32_t dtype, int64_t n, int32
     const size_t nk = (size_t)n * k;
     const int kp = std::min(p->rescore_mult * k, 128);
     // perm | lists | max(partition, leaf scratch)
-    Arena m;
-    m.take<int32_t>((size_t)T * n);
-    m.take<int32_t>((size_t)T * nk);
-    m.take<float>((size_t)T * nk);
-    const size_t fixed = m.off;
-    run_partition(x, h->plan, h->dplan, T, p->seed, nullptr, m, st);
-    const size_t pe = m.off;
-    m.off = fixed;
-    run_leaf_knn_tc(x, h->plan, h->dplan, T, nullptr, k, kp, p->precision, nullptr, nullptr, nullptr, m, st);
-    if ((r = ensure_ws(h, std::max(pe, m.off), st))) return r;
+    size_t fixed = 0;
     Arena a;
-    a.base = h->ws;
+    if ((r = take_ws(h, st, a, [&](Arena& m) {
+            m.take<int32_t>((size_t)T * n);
+            m.take<int32_t>((size_t)T * nk);
+            m.take<float>((size_t)T * nk);
+            fixed = m.off;
+            run_partition(x, h->plan, h->dplan, T, p->seed, nullptr, m, st);
+            const size_t pe = m.off;
+            m.off = fixed;
+            run_leaf_knn_tc(x, h->plan, h->dplan, T, nullptr, k, kp, p->precision, nullptr, nullptr, nullptr, m, st);
+            m.off = std::max(pe, m.off);
+            return KNNG_OK;
+        })))
+        return r;
     int32_t* perm = a.take<int32_t>((size_t)T * n);
     int32_t* li = a.take<int32_t>((size_t)T * nk);
     float* ldd = a.take<float>((size_t)T * nk);
@@ -1271,16 +1329,15 @@ int knng_build_learned(knng_handle* h, knng_mlp* m, const void* X, int32_t dtype
     learned_feature_order(q.seed, q.T, M->C, lf);
     const bool feat = mode == KNNG_PART_FEATURES || mode == KNNG_PART_FEATURES_PCA;
     XDesc xz{nullptr, KNNG_DTYPE_F32, n, M->C, M->C, true};  // the embedding as the partition's points
-    Arena m0;
-    m0.take<float>((size_t)n * M->C);
-    m0.take<uint32_t>(2 * (size_t)M->C);
-    m0.take<float>((size_t)M->C);
-    if ((r = build_pipeline(h, h->plan, h->dplan, x, q, ids, dists, m0, st, true, feat ? &lf : nullptr, true,
-                            feat ? nullptr : &xz)))
-        return r;
-    if ((r = ensure_ws(h, m0.off, st))) return r;
     Arena a;
-    a.base = h->ws;
+    if ((r = take_ws(h, st, a, [&](Arena& m) {
+            m.take<float>((size_t)n * M->C);
+            m.take<uint32_t>(2 * (size_t)M->C);
+            m.take<float>((size_t)M->C);
+            return build_pipeline(h, h->plan, h->dplan, x, q, ids, dists, m, st, true, feat ? &lf : nullptr, true,
+                                  feat ? nullptr : &xz);
+        })))
+        return r;
     float* Z = a.take<float>((size_t)n * M->C);
     uint32_t* mm = a.take<uint32_t>(2 * (size_t)M->C);
     float* frange = a.take<float>((size_t)M->C);
@@ -1315,14 +1372,15 @@ int knng_partition_learned(knng_handle* h, knng_mlp* m, const void* X, int32_t d
     LearnedFeat lf;
     lf.C = M->C;
     learned_feature_order(seed, T, M->C, lf);
-    Arena m0;
-    if (!Zout) m0.take<float>((size_t)n * M->C);
-    m0.take<uint32_t>(2 * (size_t)M->C);
-    m0.take<float>((size_t)M->C);
-    run_partition(x, h->plan, h->dplan, T, seed, nullptr, m0, st, &lf);
-    if ((r = ensure_ws(h, m0.off, st))) return r;
     Arena a;
-    a.base = h->ws;
+    if ((r = take_ws(h, st, a, [&](Arena& m) {
+            if (!Zout) m.take<float>((size_t)n * M->C);
+            m.take<uint32_t>(2 * (size_t)M->C);
+            m.take<float>((size_t)M->C);
+            run_partition(x, h->plan, h->dplan, T, seed, nullptr, m, st, &lf);
+            return KNNG_OK;
+        })))
+        return r;
     float* Z = Zout ? Zout : a.take<float>((size_t)n * M->C);
     uint32_t* mm = a.take<uint32_t>(2 * (size_t)M->C);
     float* frange = a.take<float>((size_t)M->C);
@@ -1357,7 +1415,7 @@ int knng_build_host(knng_handle* h, const void* X, int32_t dtype, int64_t n, int
         h->staging = nullptr;
         h->staging_size = 0;
         void* q = nullptr;
-        e = cudaMallocAsync(&q, need, st);
+        e = handle_alloc(h, &q, need, st);
         if (e != cudaSuccess) {
             cudaGetLastError();
             return fail(h, KNNG_ERR_OOM, "staging buffers");

@@ -89,10 +89,12 @@ struct DevPlan {
 };
 
 // Bump allocator over the handle's workspace.  With base == nullptr it only
-// measures.
+// measures.  lean: there is no memory for the stages' usual scratch; they take
+// their forms with the least of it (the same method, slower).
 struct Arena {
     char* base = nullptr;
     size_t off = 0;
+    bool lean = false;
     template <class T>
     T* take(size_t count)
     {

@@ -21,7 +21,7 @@ cudaError_t run_leaf_knn_f32(const XDesc& x, const TreePlan& P, const DevPlan& d
                              cudaStream_t st)
 {
     if (kp > kCandCap) kp = kCandCap;
-    if (leaf_rescore_staged_ok(kp, P.max_leaf)) {
+    if (!ar.lean && leaf_rescore_staged_ok(kp, P.max_leaf)) {
         // (eight more: the rescoring reads whole groups of eight)
         uint16_t* cand = ar.take<uint16_t>((size_t)T * x.n * kp + 8);
         if (!ar.base) return cudaSuccess;

@@ -123,8 +123,9 @@ cudaError_t run_leaf_knn_tc(const XDesc& x, const TreePlan& P, const DevPlan& dp
     uint8_t* qx = ar.take<uint8_t>((size_t)rows);
     if (kp > kTcCand) kp = kTcCand;
     // rows of leaves that are not exact are rescored by the staged kernel
-    // (their candidates in [rows][kp] local indices, a flag per leaf)
-    const bool staged = leaf_rescore_staged_ok(kp, P.max_leaf);
+    // (their candidates in [rows][kp] local indices, a flag per leaf); lean:
+    // by the leaf kernel itself, row by row
+    const bool staged = !ar.lean && leaf_rescore_staged_ok(kp, P.max_leaf);
     const int nleaves = (int)P.leaf_off.size() - 1;
     uint16_t* cand = staged ? ar.take<uint16_t>((size_t)T * x.n * kp + 8) : nullptr;
     uint8_t* leaf_flag = staged ? ar.take<uint8_t>((size_t)T * nleaves) : nullptr;

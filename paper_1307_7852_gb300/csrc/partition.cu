@@ -1174,8 +1174,8 @@ cudaError_t run_partition(const XDesc& x, const TreePlan& P, const DevPlan& dp, 
     int32_t* node_pos = ar.take<int32_t>((size_t)T * n);
     uint32_t* keys = ar.take<uint32_t>((size_t)T * n);
     // the directions of a run of levels at a time: as many levels as 64 MB
-    // (or one level) hold
-    int64_t dir_cap = std::max<int64_t>((int64_t)T * S_max, ((int64_t)64 << 20) / (4 * (int64_t)d_pad));
+    // (or one level; lean: one level) hold
+    int64_t dir_cap = std::max<int64_t>((int64_t)T * S_max, ar.lean ? 0 : ((int64_t)64 << 20) / (4 * (int64_t)d_pad));
     {
         int64_t all = 0;
         for (const LevelPlan& L : P.levels) all += (int64_t)T * L.nnodes;
