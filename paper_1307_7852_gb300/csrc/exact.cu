@@ -38,7 +38,7 @@
 // the origin for their spread) costs the passes beside the direct kernel: 12 %
 // at 2,048 rows and 10 queries, 3 % at 16,384 and 1,000, 1 % at 200,000.
 // 10,000 queries of 1,000,000 x 128 rows, k = 20: 788 ms with exact_knn_kernel
-// alone (seven shuffles per pair and 128 entries), 7.6 ms filtered.
+// alone (seven shuffles per pair and 128 entries), 6.9 ms filtered.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>
@@ -419,8 +419,8 @@ __host__ __device__ __forceinline__ int64_t tile_begin(int64_t total, int G, int
 // 256-column accumulators, warps 2..9 read them back: a thread has one query
 // and 128 of the tile's rows.  A tile of 128 entries a row is 1,024 cycles of
 // tensor work and about as much of the eight warps' minima, so the two
-// overlap; 10,000 queries of 1M x 128 take 3.3 ms for the minima and 4.0 ms
-// for the lists (770 and 640 TFLOP/s).
+// overlap; 10,000 queries of 1M x 128 take 3.2 ms for the minima and 3.4 ms
+// for the lists (810 and 755 TFLOP/s).
 //  kList == false: minima over 32 groups per thread, written per CTA and
 //   query tile (slot c + rt of CTA c) to mins[slot][128][64].
 //  kList == true: rows with |x^|^2 - 2 q^.x^ <= thr[query] are appended to
@@ -864,9 +864,9 @@ template <int kDT>
 std::integral_constant<int, kDT> dtype_of(const RowLoader<kDT>&);
 
 // The filtered form from 2,048 rows on: exact_knn_kernel streams all rows per
-// block, 0.51 ms at 2,048 x 128 for 10 or 1,000 queries and 3.8 ms at 16,384,
-// the filtered form 0.09 / 0.12 ms and 0.15 / 0.19 ms; smaller sets keep the
-// form that needs no scratch.  n below 2^31 - 256: row numbers of a tile stay
+// block, 0.50 ms at 2,048 x 128 for 10 or 1,000 queries and 3.8 ms at 16,384
+// for 1,000, the filtered form 0.08 and 0.13 ms; smaller sets keep the form
+// that needs no scratch.  n below 2^31 - 256: row numbers of a tile stay
 // in an int.
 bool exact_tc_ok(const XDesc& x, int nq)
 {

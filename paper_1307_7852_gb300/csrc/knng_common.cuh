@@ -908,8 +908,8 @@ __device__ __forceinline__ float dist_u8_g8(const uint8_t* X, int64_t ld, int d,
 
 // Canonical distances from a to b[0..nb) (nb <= 32): lane c < nb returns the
 // distance to b[c].  Byte rows with exact integer distances take one batch
-// of 32 (32 rows in flight per warp), other vector-aligned rows eight lanes a
-// row, the rest one distance at a time.
+// of 32 (32 rows in flight per warp); narrow rows and rows of any alignment
+// eight lanes a row (warp_canon_dist_g8), wide rows two batches of 16.
 // kForm: 0 picks by the rows here; kernels built for one form (row_form) hold
 // the code of that one only: with two, the propagation of 256-entry rows ran
 // 3 % slower.

@@ -11,7 +11,7 @@
 // Bound by FP32 issue in the products (8 rows x 8 columns a lane: 256 FMAs
 // per 16 shared loads) and by the selection.  400k x 128 rows, 4 trees,
 // leaves of 195, k' = 40: 10.1 ms with the kernel below (which re-stages the
-// leaf per 32 rows and rescores row by row from L2), 5.1 + 2.2 ms so.
+// leaf per 32 rows and rescores row by row from L2), 5.2 + 2.2 ms so.
 //
 // More candidates (leaf_knn_f32_kernel): one block per (leaf, tree).  For
 // every block of 32 rows of the leaf:

@@ -31,11 +31,11 @@ namespace knng {
 // ---------------------------------------------------------------------------
 // Tiled FP32 GEMM: C[M][N] = sum_k A(m, k) B(k, n) with A(m, k) = TA ?
 // A[k*lda + m] : A[m*lda + k] and B(k, n) = TB ? B[n*ldb + k] : B[k*ldb + n].
-// Epilogue: EPI 0 plain store, 1 = + bias[n], store pre-activation to aux and
-// GELU to C, 3 = tanh(. + bias[n]), 4 = times GELU'(aux) (the backward pass
-// through the activation), 5 = one K slice of a reduction: slice z of K
-// (kper entries) goes to C + z * (M*N + M), followed by the slice's row sums
-// of A(m, .) (the bias gradient), for grad_reduce_kernel.
+// Epilogue: EPI 1 = + bias[n], store pre-activation to aux and GELU to C, 3 =
+// tanh(. + bias[n]), 4 = times GELU'(aux) (the backward pass through the
+// activation), 5 = one K slice of a reduction: slice z of K (kper entries)
+// goes to C + z * (M*N + M), followed by the slice's row sums of A(m, .) (the
+// bias gradient), for grad_reduce_kernel.
 //
 // A thread block holds a TM x TN tile, 256 threads of (TM/16) x (TN/16)
 // entries each; the next K step of 32 is loaded into registers while the
@@ -43,8 +43,8 @@ namespace knng {
 // network's 16 or 32 outputs, where a 64-wide tile would be mostly padding.
 // The weight gradients contract over the batch (K = 8192 rows of a
 // 4,096-edge batch against 256 x 96 outputs): without the K slices 8 blocks
-// did the whole contraction (4.2 ms for the two; 23 + 11 us with slices over
-// about two blocks per SM, and 7 us to add them up).
+// did each whole contraction, most of the call's 3.4 ms; 20 + 9 us with slices
+// over about two blocks per SM, and 5 us to add them up.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ float gelu_f(float a)
 {
@@ -213,7 +213,7 @@ __global__ void sample_batch_kernel(RowLoader<kDT> L, int64_t n, const int32_t* 
 // ---------------------------------------------------------------------------
 // Loss and dL/dZ through the batch statistics.  Z: N x C rows, N = 2B.
 // Four passes over blocks of kLossRows rows (one block did it all before:
-// 0.70 ms of an 8192 x 16 batch, now 56 us in all): column sums; centred second
+// 0.70 ms of an 8192 x 16 batch, now 49 us in all): column sums; centred second
 // moments and the pairs' differences; the statistics and the loss (one
 // block, sums of the row blocks in FP64); the gradient.
 //   K = corr, S = (z - mean) / sqrt(var + eps), dS = (2/N) S G with
