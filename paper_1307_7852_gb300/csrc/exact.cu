@@ -225,6 +225,7 @@ struct ExactStats {
     uint32_t max_nrm;
     uint32_t bad;
     uint32_t nfar;
+    uint32_t gave_up;  // a bounded wait of this call's passes
     int32_t far[2 * kFarRows];
     uint32_t nrm_hist[256];
     uint32_t err_hist[256];
@@ -434,7 +435,7 @@ __host__ __device__ __forceinline__ int64_t tile_begin(int64_t total, int G, int
 template <bool kList, bool kPoll>
 __global__ void __launch_bounds__(kGramThreads, 1) exact_gram_kernel(
     const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUtensorMap bmap, int nK, int RT, int CT,
-    bool a_stays, const float* __restrict__ nrm, const ExactStats* __restrict__ stats, float* __restrict__ mins,
+    bool a_stays, const float* __restrict__ nrm, ExactStats* __restrict__ stats, float* __restrict__ mins,
     const float* __restrict__ thr, int* __restrict__ counts, int32_t* __restrict__ lists, long long limit, int* err)
 {
     if (stats->bad) return;
@@ -474,6 +475,7 @@ __global__ void __launch_bounds__(kGramThreads, 1) exact_gram_kernel(
     const int64_t g0 = tile_begin(total, gridDim.x, blockIdx.x), g1 = tile_begin(total, gridDim.x, blockIdx.x + 1);
     auto give_up = [&]() {
         abort_flag = 1;
+        atomicExch(&stats->gave_up, 1u);
         atomicExch(err, 1);
     };
     // a bounded wait that also ends when another warp gave up
@@ -779,8 +781,8 @@ __global__ void __launch_bounds__(256) exact_bound_kernel(int64_t n, int d, int 
 template <int kDT>
 __global__ void __launch_bounds__(kRescoreWarps * 32) exact_rescore_kernel(
     RowLoader<kDT> L, int64_t n, const int32_t* __restrict__ queries, int nq, int k, const int* __restrict__ counts,
-    const int32_t* __restrict__ lists, uint8_t* __restrict__ need, const int* __restrict__ err,
-    int32_t* __restrict__ out_ids, float* __restrict__ out_d)
+    const int32_t* __restrict__ lists, uint8_t* __restrict__ need,
+    const ExactStats* __restrict__ stats, int32_t* __restrict__ out_ids, float* __restrict__ out_d)
 {
     __shared__ uint64_t buf_all[kRescoreWarps][kListMax];
     __shared__ uint32_t hist_all[kRescoreWarps][256];
@@ -792,7 +794,7 @@ __global__ void __launch_bounds__(kRescoreWarps * 32) exact_rescore_kernel(
     if (need[qi]) return;
     const int cnt = counts[qi];
     // (a wait that gave up leaves rows unlisted: the direct kernel answers)
-    if (cnt > kListMax || *err != 0) {
+    if (cnt > kListMax || stats->gave_up) {
         if (lane == 0) need[qi] = 1;
         return;
     }
@@ -949,7 +951,7 @@ cudaError_t run_exact_knn_tc(const XDesc& x, const int32_t* queries, int nq, int
         note_launches(3);
         typed([&](auto rl) {
             exact_rescore_kernel<<<(cq + kRescoreWarps - 1) / kRescoreWarps, kRescoreWarps * 32, 0, st>>>(
-                rl, x.n, qs, cq, k, counts, lists, need, err, oi, od);
+                rl, x.n, qs, cq, k, counts, lists, need, stats, oi, od);
             note_launches(1);
         });
         e = run_exact_knn(x, qs, cq, k, oi, od, st, need);

@@ -37,3 +37,21 @@ def test_waits_run_out_and_the_lists_stay_right(n, d, nq):
     gi, gd = k.knng_exact_knn(Xd, qd, 9, h=h)
     k.knng_sync(h)
     assert_lists_exact(host(gi), host(gd), oi, od)
+
+
+def test_an_earlier_calls_timeout_leaves_the_filter_on():
+    # the handle's error word stays set until knng_sync reads it
+    from test_gpu_exact_cost import best_ms, call_and_direct, normal_rows
+    k = knng()
+    X = normal_rows(60000, 64, 5)
+    q = torch.arange(1000, dtype=torch.int32, device="cuda") * 60
+    direct = call_and_direct(X, q, 10)[1]
+    h = k.Handle(0)
+    perm = k.knng_partition(X, 1, 128, 3, h=h)
+    k.knng_sync(h)
+    k.knng_set_wait_limit(8, h)
+    k.knng_leaf_knn(X, 1, 128, perm, 10, k.PREC_BF16, 2, h=h)
+    k.knng_set_wait_limit(0, h)
+    assert best_ms(lambda: k.knng_exact_knn(X, q, 10, h=h)) < 0.5 * direct
+    with pytest.raises(k.KnngError):
+        k.knng_sync(h)
