@@ -645,7 +645,9 @@ __global__ void __launch_bounds__(kTcThreads, PER == 16 ? 1 : 2) leaf_tc_kernel(
                 for (int e = 0; e < 32; e += 4) {
                     const bool room = at <= at0 + (kListCap - 4) * kStep;
                     ovf |= !room;
-                    const float lim = room ? tau : -kInf;
+                    // (NaN: nothing passes, also not the -inf of a row past the
+                    // leaf, whose operand may be another leaf's infinite row)
+                    const float lim = room ? tau : __int_as_float(0x7fffffff);
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
                         if (dv[e + q] <= lim) {
