@@ -379,7 +379,10 @@ __global__ void __launch_bounds__(kNT, CT > 8 ? 1 : 2) leaf_cand_f32_kernel(RowL
 #pragma unroll
         for (int c = 0; c < CT; ++c) {
             const int col = lane + 32 * c;
-            const uint32_t o = ord_key(ni + nrm[col] - 2.f * acc[r][c]);
+            const float dist = ni + nrm[col] - 2.f * acc[r][c];
+            // (a distance that is not a number comes after all others, whatever
+            // its sign bit: as a key it came before them)
+            const uint32_t o = dist == dist ? ord_key(dist) : 0xFFFFFFFEu;
             h[c] = (col < m && col != row) ? min(o, 0xFFFFFFFEu) : 0xFFFFFFFFu;
         }
         warp_pick_columns<CT>(h, want, scr, cand + (rowbase + row) * kp);

@@ -16,7 +16,7 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("precision", [0, 1, 2])
 @pytest.mark.parametrize("dtype", [torch.float32, torch.float16])
-@pytest.mark.parametrize("g,k", [(64, 5), (100, 20), (256, 24)])
+@pytest.mark.parametrize("g,k", [(64, 5), (100, 20), (256, 24), (500, 12), (200, 40)])
 def test_finite_rows_keep_their_lists(precision, dtype, g, k):
     rng = np.random.default_rng(g + k)
     n, d = 3000, 24
